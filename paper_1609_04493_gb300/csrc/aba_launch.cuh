@@ -233,6 +233,33 @@ bool aba_use_tri(int n, int B, int flags, bool ext)
     return !ext && B <= 2048;
 }
 
+// Three lanes per instance (aba_trio.cuh): by flag, else for FP32 data with
+// double-float updates (also where the two- or three-warp form is asked for, which
+// it supersedes there) while the batch is resident at once, which is what the
+// split is for: four blocks per SM (thirty instances each, or twenty with the
+// double-float bias sweeps, where two such waves still win). Times in us on
+// GB300, the mapping taken otherwise / three lanes: n = 7: 17.6 / 14.9 at B = 1024, 34.9 / 23.7 at
+// 18240, 35.7 / 38.1 at 24000; n = 64: 346 / 218 at 18240, 360 / 355 at 24000, 352 /
+// 440 at 32768; n = 100: 822 / 708 at 16384, 990 / 852 at 24000, 938 / 1197 at
+// 32768. Below three links nothing is left to split (n = 2: 5.2 / 5.3 at B = 64,
+// 7.5 / 8.0 at 16384).
+inline bool aba_use_trio(const rd_model *m, int B, int flags, bool ext)
+{
+    if (flags & RD_ABA_THREE_LANES) return true;
+    if (flags & (RD_ABA_THREAD_PER_INSTANCE | RD_ABA_WARP_PER_INSTANCE | RD_ABA_JOINT_FRAMES |
+                 RD_ABA_SCANS_IN_DTYPE | RD_ABA_FP64_UPDATE | RD_ABA_TEST_WITHHOLD))
+        return false;
+    static std::atomic<int> sms[64];
+    std::atomic<int> &slot = sms[m->device & 63];
+    int count = slot.load();
+    if (!count) {
+        if (cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, m->device) != cudaSuccess)
+            return false;
+        slot.store(count);
+    }
+    return m->n >= 3 && (long long)B <= (ext ? 160LL : 120LL) * count;
+}
+
 template <typename T>
 int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const void *tau,
                  void *qdd, int *status, void *ws, size_t ws_bytes, const double *base18,
@@ -247,18 +274,27 @@ int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const 
     if (!aba_aligned16(ws)) return rd_fail(RD_ERR_ARG, "aba_batch: workspace not 16-byte aligned");
     {
         const int maps = !!(flags & RD_ABA_WARP_PER_INSTANCE) + !!(flags & RD_ABA_TWO_WARPS) +
-                         !!(flags & RD_ABA_THREE_WARPS) + !!(flags & RD_ABA_THREAD_PER_INSTANCE);
+                         !!(flags & RD_ABA_THREE_WARPS) + !!(flags & RD_ABA_THREE_LANES) +
+                         !!(flags & RD_ABA_THREAD_PER_INSTANCE);
         if (maps > 1 ||
-            ((flags & (RD_ABA_WARP_PER_INSTANCE | RD_ABA_TWO_WARPS | RD_ABA_THREE_WARPS)) &&
+            ((flags & (RD_ABA_WARP_PER_INSTANCE | RD_ABA_TWO_WARPS | RD_ABA_THREE_WARPS |
+                       RD_ABA_THREE_LANES)) &&
              (flags & (RD_ABA_JOINT_FRAMES | RD_ABA_SCANS_IN_DTYPE))))
             return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_WARP_PER_INSTANCE, RD_ABA_TWO_WARPS, "
-                                       "RD_ABA_THREE_WARPS and RD_ABA_THREAD_PER_INSTANCE exclude "
-                                       "one another, and the first three RD_ABA_JOINT_FRAMES and "
-                                       "RD_ABA_SCANS_IN_DTYPE");
+                                       "RD_ABA_THREE_WARPS, RD_ABA_THREE_LANES and "
+                                       "RD_ABA_THREAD_PER_INSTANCE exclude one another, and the "
+                                       "first four RD_ABA_JOINT_FRAMES and RD_ABA_SCANS_IN_DTYPE");
+        if ((flags & RD_ABA_THREE_LANES) && (sizeof(T) != 4 || (flags & RD_ABA_FP64_UPDATE)))
+            return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_THREE_LANES takes RD_F32 data with "
+                                       "double-float updates");
     }
     const bool withhold = (flags & RD_ABA_TEST_WITHHOLD) != 0;
     if (withhold && !(flags & RD_ABA_TWO_WARPS))
         return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_TEST_WITHHOLD needs RD_ABA_TWO_WARPS");
+    if constexpr (sizeof(T) == 4) {
+        if (aba_use_trio(m, B, flags, ext))
+            return rd_aba_trio_f32(m, B, q, qd, tau, qdd, status, ws, base18, ext, s);
+    }
     if (aba_use_tri<T>(m->n, B, flags, ext)) {
         if constexpr (sizeof(T) == 4)
             return rd_aba_tri_f32(m, B, q, qd, tau, qdd, status, ws, base18,

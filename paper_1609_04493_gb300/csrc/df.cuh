@@ -77,9 +77,110 @@ __device__ __forceinline__ DF fma(DF x, DF y, DF z)
 __device__ __forceinline__ DF &operator+=(DF &x, DF y) { return x = x + y; }
 __device__ __forceinline__ DF &operator-=(DF &x, DF y) { return x = x - y; }
 
+// ---- sums formed as one: the errors of the products and of the partial sums
+// of the high parts are added up beside the high part. Error: a
+// few units of 2^-48 times the sum of the terms' magnitudes, no more than the
+// same sum as a chain of multiply-adds, for fewer instructions (two products: 16
+// against 22; three: 28 against 37; four terms: 24 against 33).
+
+// high part and error of x y; of c y for a plain float c
+__device__ __forceinline__ DF df_prod(DF x, DF y)
+{
+    const float p = x.hi * y.hi;
+    return DF(p, fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, fmaf(x.hi, y.hi, -p))));
+}
+__device__ __forceinline__ DF df_prod(float c, DF y)
+{
+    const float p = c * y.hi;
+    return DF(p, fmaf(c, y.lo, fmaf(c, y.hi, -p)));
+}
+
+// The _raw forms leave the result unnormalised: hi is the rounded sum of the high
+// parts, lo every error and low part. As an operand of a further sum of products
+// it is as good (the neglected lo lo is 2^-48 of the magnitudes that went into
+// it, as the value's own error is); what is carried on from link to link is
+// renormalised (df_renorm).
+__device__ __forceinline__ DF df_renorm(DF x) { return df_fast_two_sum(x.hi, x.lo); }
+
+// x0 y0 + x1 y1 (S: DF or float)
+template <typename S>
+__device__ __forceinline__ DF ddot2_raw(S x0, DF y0, S x1, DF y1)
+{
+    const DF p = df_prod(x0, y0), r = df_prod(x1, y1);
+    const DF s = df_two_sum(p.hi, r.hi);
+    return DF(s.hi, s.lo + (p.lo + r.lo));
+}
+
+__device__ __forceinline__ DF ddot3_raw(DF x0, DF y0, DF x1, DF y1, DF x2, DF y2)
+{
+    const DF p = df_prod(x0, y0), r = df_prod(x1, y1), t = df_prod(x2, y2);
+    const DF s = df_two_sum(p.hi, r.hi);
+    const DF u = df_two_sum(s.hi, t.hi);
+    return DF(u.hi, (s.lo + u.lo) + (p.lo + r.lo + t.lo));
+}
+
+// x y + z
+__device__ __forceinline__ DF dfma_raw(DF x, DF y, DF z)
+{
+    const DF p = df_prod(x, y);
+    const DF s = df_two_sum(p.hi, z.hi);
+    return DF(s.hi, s.lo + (p.lo + z.lo));
+}
+
+__device__ __forceinline__ DF dsum2_raw(DF x, DF y)
+{
+    const DF s = df_two_sum(x.hi, y.hi);
+    return DF(s.hi, s.lo + (x.lo + y.lo));
+}
+
+__device__ __forceinline__ DF dsum3_raw(DF x, DF y, DF z)
+{
+    const DF s = df_two_sum(x.hi, y.hi);
+    const DF u = df_two_sum(s.hi, z.hi);
+    return DF(u.hi, (s.lo + u.lo) + (x.lo + y.lo + z.lo));
+}
+
+__device__ __forceinline__ DF dsum4_raw(DF x, DF y, DF z, DF w)
+{
+    const DF s = df_two_sum(x.hi, y.hi), t = df_two_sum(z.hi, w.hi);
+    const DF u = df_two_sum(s.hi, t.hi);
+    return DF(u.hi, (s.lo + t.lo + u.lo) + ((x.lo + y.lo) + (z.lo + w.lo)));
+}
+
+__device__ __forceinline__ DF dmul_raw(DF x, DF y) { return df_prod(x, y); }
+__device__ __forceinline__ DF dmul_raw(float c, DF y) { return df_prod(c, y); }
+
 }  // namespace dfloat
+using dfloat::ddot2_raw;
+using dfloat::ddot3_raw;
 using dfloat::DF;
+using dfloat::df_renorm;
 using dfloat::df_two_sum;
+using dfloat::dfma_raw;
+using dfloat::dmul_raw;
+using dfloat::dsum2_raw;
+using dfloat::dsum3_raw;
+using dfloat::dsum4_raw;
+
+// the same in FP64
+__device__ __forceinline__ double df_renorm(double x) { return x; }
+__device__ __forceinline__ double ddot2_raw(double x0, double y0, double x1, double y1)
+{
+    return fma(x0, y0, x1 * y1);
+}
+__device__ __forceinline__ double ddot3_raw(double x0, double y0, double x1, double y1, double x2,
+                                            double y2)
+{
+    return fma(x0, y0, fma(x1, y1, x2 * y2));
+}
+__device__ __forceinline__ double dfma_raw(double x, double y, double z) { return fma(x, y, z); }
+__device__ __forceinline__ double dsum2_raw(double x, double y) { return x + y; }
+__device__ __forceinline__ double dsum3_raw(double x, double y, double z) { return (x + y) + z; }
+__device__ __forceinline__ double dsum4_raw(double x, double y, double z, double w)
+{
+    return (x + y) + (z + w);
+}
+__device__ __forceinline__ double dmul_raw(double x, double y) { return x * y; }
 
 // ---- helpers overloaded for double and DF
 
@@ -128,6 +229,12 @@ __device__ __forceinline__ D dsub_exact(T a, T b)
     return DSub<D>::sub(a, b);
 }
 
+// the value of lane src
+__device__ __forceinline__ DF df_shfl(DF x, int src)
+{
+    return DF(__shfl_sync(0xffffffffu, x.hi, src), __shfl_sync(0xffffffffu, x.lo, src));
+}
+
 // conversions between the data types (float, double) and D
 template <typename To>
 struct DCvt;
@@ -153,6 +260,28 @@ template <typename To, typename From>
 __device__ __forceinline__ To dcvt(From x)
 {
     return DCvt<To>::from(x);
+}
+
+// A plain factor (the sine or cosine of a joint angle) beside values of type D:
+// an FP32 factor stays a float next to double-floats (its products take one
+// multiply-add less), and becomes a double next to doubles.
+template <typename D>
+struct DScalar;
+template <>
+struct DScalar<double> {
+    __device__ __forceinline__ static double from(float x) { return (double)x; }
+    __device__ __forceinline__ static double from(double x) { return x; }
+    __device__ __forceinline__ static double from(DF x) { return (double)x.hi + (double)x.lo; }
+};
+template <>
+struct DScalar<DF> {
+    __device__ __forceinline__ static float from(float x) { return x; }
+    __device__ __forceinline__ static DF from(DF x) { return x; }
+};
+template <typename D, typename From>
+__device__ __forceinline__ auto dscalar(From x)
+{
+    return DScalar<D>::from(x);
 }
 
 // nearest double-float of a double (host side: records are split once;
