@@ -439,7 +439,10 @@ enum rd_schedule {
  * arithmetic (as RD_ABA_FP64_UPDATE for aba_batch). */
 #define RD_FLEET_FP64_UPDATE 0x10
 /* Tuning word for RD_SCHED_PERSISTENT: threads per CTA = 2^t, CTAs per SM = c
- * (0 = library default: 128 threads, 4 CTAs per SM). */
+ * (0 = library default: 4 CTAs per SM of 128 threads, or of 64 where an RD_F32 plan
+ * has few requests). Forward-dynamics requests of RD_F32 plans with double-float
+ * updates run three lanes per request (as RD_ABA_THREE_LANES), ten per pair of
+ * warps. */
 #define RD_FLEET_TUNE(log2_threads, ctas_per_sm) (((log2_threads) << 8) | (ctas_per_sm))
 /* OR-ed into the tune word of the persistent schedule: groups of 32 sorted
  * requests that start with a forward-dynamics chain of at least min_links links

@@ -416,6 +416,7 @@ __device__ __forceinline__ int aba_trio_solve(const D *__restrict__ sd, int n, i
         const int ii = !RAGGED || in ? i : n - 1;
         const D *r = sd + ii * kAbaDh64;
         const int u = nmax - 1 - i;
+        if (RAGGED && ii > 0) prefetch_l1(sd + (ii - 1) * kAbaDh64);
         const SolveIn cur = take(u, false);
         fetch(u + kTrioRing - 1, i - (kTrioRing - 1), false);
         const S c = cur.c, s = cur.s;
@@ -458,6 +459,7 @@ __device__ __forceinline__ int aba_trio_solve(const D *__restrict__ sd, int n, i
         const bool in = !RAGGED || i < n;
         const int ii = !RAGGED || in ? i : n - 1;
         const D *r = sd + ii * kAbaDh64;
+        if (RAGGED && ii + 1 < n) prefetch_l1(sd + (ii + 1) * kAbaDh64);
         const SolveIn cur = take(i, true);
         fetch(i + kTrioRing - 1, i + kTrioRing - 1, true);
         const S c = cur.c, s = cur.s;
@@ -487,8 +489,8 @@ __device__ __forceinline__ int aba_trio_solve(const D *__restrict__ sd, int n, i
 }
 
 // The bias sweeps of one instance in T, one thread: those of aba_pair.cuh's warp
-// Z, up to tau_hat.
-template <typename T, typename D, int TRIG>
+// Z, up to tau_hat. PF: constants in global memory, prefetched a link ahead.
+template <typename T, typename D, int TRIG, bool PF = false>
 __device__ __forceinline__ void aba_trio_bias(const T *__restrict__ sc, int n,
                                               const T *__restrict__ qr,
                                               const T *__restrict__ qdr,
@@ -502,6 +504,7 @@ __device__ __forceinline__ void aba_trio_bias(const T *__restrict__ sc, int n,
     x.al = mk3(base.dV0[3], base.dV0[4], base.dV0[5]);
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
+        if (PF && i + 1 < n) prefetch_l1(sc + (i + 1) * kDhConsts);
         T s, c;
         DhLink<T> L;
         load_dh(sc + i * kDhConsts, L);
@@ -633,6 +636,7 @@ __device__ __forceinline__ void aba_trio_bias_df(const DF *__restrict__ sdf, int
         const DF *r = sdf + ii * kAbaDh64;
         const DF fh = bias_get<DF>(ws, B, b, ii, k), nh = bias_get<DF>(ws, B, b, ii, 3 + k);
         const DF c = bias_get<DF>(ws, B, b, ii, 6), s = bias_get<DF>(ws, B, b, ii, 7);
+        if (RAGGED && ii > 0) prefetch_l1(sdf + (ii - 1) * kAbaDh64);
         const DF ca = r[0], sa = r[1];
         const DF nb1 = r[2 + k1], nb2 = r[2 + k2];
         const float tau = __ldg(taur + ii);

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <atomic>
+#include <cstdint>
 #include <new>
 #include <numeric>
 #include <type_traits>
@@ -46,6 +47,10 @@ struct rd_plan {
     // starts it (0 when it starts with inverse dynamics), for the two-warp
     // schedule's threshold
     std::vector<int> group_fd_n;
+    // three-lane forward dynamics (FP32 plans): the number of forward-dynamics
+    // requests, and the workspace per ten sorted positions
+    int fd_count = 0;
+    long long *unit_ws = nullptr, *unit_wz = nullptr;
     unsigned char *ws = nullptr;
     size_t ws_bytes = 0;
     int sms = 0;
@@ -162,6 +167,8 @@ extern "C" void rd_plan_destroy(rd_plan *p)
     cudaFree(p->req_off);
     cudaFree(p->group_ws);
     cudaFree(p->group_wz);
+    cudaFree(p->unit_ws);
+    cudaFree(p->unit_wz);
     cudaFree(p->ws);
     for (int k = 0; k < rd_plan::kSide; ++k) {
         if (p->side[k]) cudaStreamDestroy(p->side[k]);
@@ -222,8 +229,26 @@ extern "C" int rd_plan_create(const rd_fleet *f, int R, const int *robot, const 
         gwz[g] = (long long)ws;
         ws += (nmax * 8 * 32 * 8 + 255) & ~(size_t)255;
     }
+    // the same buffer laid out for the three-lane body: per ten sorted positions,
+    // with double-float bias state where the first position's group asks for it
+    // (the positions are sorted, so it is the unit's longest chain)
+    int fd_count = 0;
+    while (fd_count < R && kind[order[fd_count]] == RD_REQ_FD) ++fd_count;
+    std::vector<long long> uws, uwz;
+    if (dtype == RD_F32) {
+        size_t at = 0;
+        for (int k = 0; k < fd_count; k += rdyn::kTrioPerWarp) {
+            const size_t nmax = (size_t)f->n[robot[order[k]]];
+            uws.push_back((long long)at);
+            at += (nmax * ((k >> 5) < ext_groups ? 16 : 10) * rdyn::kTrioPerWarp * 4 + 255) & ~(size_t)255;
+            uwz.push_back((long long)at);
+            at += (nmax * 8 * rdyn::kTrioPerWarp * 8 + 255) & ~(size_t)255;
+        }
+        ws = std::max(ws, at);
+    }
     rd_plan *p = new (std::nothrow) rd_plan();
     if (!p) return rd_fail(RD_ERR_ALLOC, "rd_plan_create: host allocation failed");
+    p->fd_count = fd_count;
     p->fleet = f;
     p->dtype = dtype;
     p->R = R;
@@ -243,6 +268,8 @@ extern "C" int rd_plan_create(const rd_fleet *f, int R, const int *robot, const 
     if (e == cudaSuccess) e = upload(&p->req_off, off.data(), off.size());
     if (e == cudaSuccess) e = upload(&p->group_ws, gws.data(), gws.size());
     if (e == cudaSuccess) e = upload(&p->group_wz, gwz.data(), gwz.size());
+    if (e == cudaSuccess) e = upload(&p->unit_ws, uws.data(), uws.size());
+    if (e == cudaSuccess) e = upload(&p->unit_wz, uwz.data(), uwz.size());
     if (e == cudaSuccess) e = cudaMalloc(&p->counter, 2 * sizeof(int));  // + the pair counter
     if (e == cudaSuccess) e = cudaMalloc(&p->ws, std::max<size_t>(ws, 16));
     p->ws_bytes = ws;
@@ -299,6 +326,9 @@ int run_fleet(const rd_plan *p, const void *q, const void *qd, const void *in2, 
     a.ext_groups = p->ext_groups;
     a.pair_groups = 0;
     a.pair_counter = p->counter + 1;
+    a.fd_count = p->fd_count;
+    a.unit_ws = p->unit_ws;
+    a.unit_wz = p->unit_wz;
     a.robot_n = f->robot_n;
     a.robot_link = f->robot_link;
     a.order = p->order;
@@ -351,9 +381,33 @@ int run_fleet(const rd_plan *p, const void *q, const void *qd, const void *in2, 
         int per_sm = tune & 0xff ? tune & 0xff : 4;
         if (threads < 32 || threads > 1024)
             return rd_fail(RD_ERR_ARG, "fleet_batch: %d threads per block", threads);
-        e = cudaMemsetAsync(p->counter, 0, sizeof(int), s);
+        e = cudaMemsetAsync(p->counter, 0, 2 * sizeof(int), s);
         if (e != cudaSuccess) return rd_cuda_fail(e, "fleet_batch: counter reset");
-        rdyn::fleet_persistent_kernel<T, D><<<p->sms * per_sm, threads, 0, s>>>(a);
+        if constexpr (std::is_same<D, rdyn::DF>::value) {
+            // By default one pair of warps per block where every unit then has
+            // a pair at once and the inverse-dynamics requests are few: the other
+            // two warps would only take issue slots from the longest chains, which
+            // set the time (us, 128 threads / 64: 20 000 requests of 6..100 links 377 /
+            // 335, of 6..64 184 / 158, 4000 of 8..40 91 / 85; 100 000 594 / 792, where
+            // neither holds).
+            const int units = (p->fd_count + rdyn::kTrioPerWarp - 1) / rdyn::kTrioPerWarp;
+            const int grid = p->sms * per_sm, id_groups = (p->R - p->fd_count + 31) / 32;
+            if (!((tune >> 8) & 0xff) && units && units <= grid && id_groups <= 2 * grid) threads = 64;
+            const int pairs = std::min(std::max(threads / 64, 1), rdyn::kFleetTrioPairs);
+            const size_t smem = pairs * sizeof(rdyn::FleetTrioShared);
+            static std::atomic<uint64_t> configured{0};
+            const uint64_t bit = 1ull << (f->device & 63);
+            if (!(configured.load() & bit)) {
+                e = cudaFuncSetAttribute(rdyn::fleet_trio_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         rdyn::kFleetTrioPairs * (int)sizeof(rdyn::FleetTrioShared));
+                if (e != cudaSuccess) return rd_cuda_fail(e, "cudaFuncSetAttribute");
+                configured.fetch_or(bit);
+            }
+            rdyn::fleet_trio_kernel<<<p->sms * per_sm, threads, smem, s>>>(a);
+        } else {
+            rdyn::fleet_persistent_kernel<T, D><<<p->sms * per_sm, threads, 0, s>>>(a);
+        }
     } else if (schedule == RD_SCHED_PER_GROUP) {
         // one launch per group, spread over side streams that fork from and
         // join back into the caller's stream (so groups can run concurrently)
@@ -364,7 +418,18 @@ int run_fleet(const rd_plan *p, const void *q, const void *qd, const void *in2, 
         int k = 0;
         for (const auto &g : p->groups) {
             const int len = g.second - g.first;
-            rdyn::fleet_range_kernel<T, D><<<(len + 127) / 128, 128, 0, p->side[k]>>>(a, g.first, g.second);
+            if constexpr (std::is_same<D, rdyn::DF>::value) {
+                if (g.first < p->fd_count) {
+                    const int units = (g.second - 1) / rdyn::kTrioPerWarp - g.first / rdyn::kTrioPerWarp + 1;
+                    rdyn::fleet_trio_range_kernel<<<units, 64, 0, p->side[k]>>>(a, g.first, g.second);
+                } else {
+                    rdyn::fleet_id_range_kernel<T, D><<<(len + 127) / 128, 128, 0, p->side[k]>>>(
+                        a, g.first, g.second);
+                }
+            } else {
+                rdyn::fleet_range_kernel<T, D><<<(len + 127) / 128, 128, 0, p->side[k]>>>(
+                    a, g.first, g.second);
+            }
             k = (k + 1) % rd_plan::kSide;
         }
         for (int j = 0; j < rd_plan::kSide && e == cudaSuccess; ++j) {
