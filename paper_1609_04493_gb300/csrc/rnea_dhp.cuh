@@ -15,7 +15,7 @@
 // * Trigonometry (FP32). The default evaluates sin/cos of q_i + theta0_i with
 //   the FMA-pipe polynomials of trig_poly.cuh (error under one ulp); TRIG = 1
 //   selects the special-function-unit approximation (RD_FLAG_FAST_TRIG). FP64
-//   uses the library's sincos.
+//   takes trig_fixed.cuh.
 // For chains of at most NMAX links, n % 4 == 0 and 16-byte aligned rows.
 #pragma once
 #include "rnea_dh.cuh"
@@ -33,7 +33,7 @@ enum DhTrig { kTrigPoly = 0, kTrigSfu = 1 };
 template <typename T, int TRIG>
 __device__ __forceinline__ void dh_trig(T x, T *s, T *c)
 {
-    if constexpr (sizeof(T) == 8) sincos(x, s, c);
+    if constexpr (sizeof(T) == 8) sincos_fixed(x, s, c);
     else if constexpr (TRIG == kTrigSfu) sincos_fast(x, s, c);
     else sincos_poly(x, s, c);
 }

@@ -16,6 +16,7 @@
 #include <cuda_pipeline_primitives.h>
 
 #include "spatial.cuh"
+#include "trig_fixed.cuh"
 
 namespace rdyn {
 
@@ -29,7 +30,7 @@ struct BaseParams {
 enum StateMode { kStore = 0, kRecompute = 1, kRecomputeCS = 2 };
 
 __device__ __forceinline__ void sincos_t(float x, float *s, float *c) { sincosf(x, s, c); }
-__device__ __forceinline__ void sincos_t(double x, double *s, double *c) { sincos(x, s, c); }
+__device__ __forceinline__ void sincos_t(double x, double *s, double *c) { sincos_fixed(x, s, c); }
 
 // Link constants from shared memory with 16-byte loads.
 template <typename T>
