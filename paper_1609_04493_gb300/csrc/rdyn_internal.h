@@ -61,6 +61,10 @@ void rd_convert_base_dh(const rd_model *m, const double in18[18], double out[18]
 int rd_build_dh(int n, const std::vector<double> &c64, std::vector<double> &dh64, double GBR[9],
                 double GBp[3], double *phi_last);
 void rd_build_aba64(int n, const std::vector<double> &dh64, std::vector<double> &out);
+// kfull of rd_rnea_dh_f64 for the rows that AUTO sends there, where
+// rd_rnea_dhp_f64_fits says so
+constexpr int RD_DHP_AUTO_F64 = -2;
+bool rd_rnea_dhp_f64_fits(const rd_model *m);
 int rd_rnea_dh_f32(const rd_model *m, int B, const void *q, const void *qd, const void *qdd,
                    void *tau, const double *base18, int stored, int block, int fast,
                    int kfull, int tmem, int reg_links, int stages, cudaStream_t s);

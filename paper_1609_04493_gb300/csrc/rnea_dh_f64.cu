@@ -7,3 +7,5 @@ int rd_rnea_dh_f64(const rd_model *m, int B, const void *q, const void *qd, cons
 {
     return rdyn::dh_launch<double>(m, B, q, qd, qdd, tau, base18, stored != 0, block, false, kfull, tmem != 0, reg_links, stages, s);
 }
+
+bool rd_rnea_dhp_f64_fits(const rd_model *m) { return rdyn::dhp_f64_k<double>(m) >= 0; }

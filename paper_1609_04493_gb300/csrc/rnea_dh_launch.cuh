@@ -114,7 +114,13 @@ int launch_dhp_k(const rd_model *m, int K, int B, const void *q, const void *qd,
         configured.fetch_or(bit);
     }
     DhParamConsts<T, NMAX> pc;
-    for (int k = 0; k < m->n * kDhConsts; ++k) pc.c[k] = (T)m->host_dh64[k];
+    for (int i = 0; i < m->n; ++i) {
+        const double *h = &m->host_dh64[(size_t)i * kDhConsts];
+        double S[6];
+        dh_second_moments(h + 10, S);
+        for (int k = 0; k < 10; ++k) pc.c[i * kDhConsts + k] = (T)h[k];
+        for (int k = 0; k < 6; ++k) pc.c[i * kDhConsts + 10 + k] = (T)S[k];
+    }
     for (int k = m->n * kDhConsts; k < NMAX * kDhConsts; ++k) pc.c[k] = T(0);
     const unsigned grid = (unsigned)((B + BLOCK - 1) / BLOCK);
     rd_note_rnea(RD_RNEA_KERNEL_DH_PARAM, BLOCK, K, RL, STG);
@@ -196,7 +202,9 @@ bool dhp_eligible(const rd_model *m, const void *q, const void *qd, const void *
 // 18.54 / 17.39 (8, two); 32: 21.78 / 20.25 (8, three; two: 20.96). Where RL =
 // 4 with the two-chunk ring holds the whole batch in half a wave it leads (n =
 // 16, B = 16384: 4.09 against 4.50 with 8; n = 32, B = 16384: 6.75 against
-// 7.14); near a full wave 8 does (n = 16, B = 65536: 9.18 against 9.39). 12 and
+// 7.14); near a full wave 8 does (n = 16, B = 65536: 9.18 against 9.39). (Those were
+// taken with the recursion by spatial velocities; by origin accelerations, kin_forward,
+// the same layouts take n = 8: 5.00, 16: 8.47, 28: 14.9, 32: 18.4.) 12 and
 // 16 register links never led: more blocks per SM, longer unrolled code.
 template <int TRIG>
 void dhp_default_kr(const rd_model *m, int B, int &K, int &RL, int &stages)
@@ -291,6 +299,39 @@ int launch_dhp(const rd_model *m, int block, int K, int B, const void *q, const 
                    : launch_dhp_b<T, 32, kTrigPoly>(m, block, K, B, q, qd, qdd, tau, base, smem, s);
     return sfu ? launch_dhp_b<T, 128, kTrigSfu>(m, block, K, B, q, qd, qdd, tau, base, smem, s)
                : launch_dhp_b<T, 128, kTrigPoly>(m, block, K, B, q, qd, qdd, tau, base, smem, s);
+}
+
+// FP64 by AUTO: the largest K whose state leaves four 32-thread blocks per SM, the
+// first eight links' state in registers (RL = 8) and a ring of two chunks; -1 where
+// not even the cosines and sines fit (n > 108). One warp per scheduler keeps the FP64
+// unit as busy as it gets (one DFMA a warp takes 64 cycles alone and 76 beside
+// three others, whatever the dependences), so what counts is the instructions: 122 a
+// stored link, 178 a re-derived one, where the joint-frame kernels took 176 and more.
+// us, joint frames / now: B = 65536: n = 8: 190 / 139, 16: 380 / 282, 32: 783 / 609,
+// 48: 1457 / 1058, 64: 2022 / 1545; B = 16384: n = 100: 901 / 650.
+template <typename T>
+int dhp_f64_k(const rd_model *m)
+{
+    static std::atomic<int> smem_sm[64];
+    const int d = m->device & 63, n = m->n;
+    if (smem_sm[d].load() == 0)
+        smem_sm[d].store(dh_device_attr(m->device, cudaDevAttrMaxSharedMemoryPerMultiprocessor, 100 * 1024));
+    const size_t limit = (size_t)smem_sm[d].load() / 4 - 1024;  // less the block's reserve
+    const int RL = n < 8 ? 0 : 8;
+    int K = n;
+    while (K >= RL && dhp_smem_per_thread<T>(n, K, RL, 2) * 32 > limit) K -= 4;
+    return K >= RL ? K : -1;
+}
+
+template <typename T>
+int launch_dhp_f64(const rd_model *m, int K, int B, const void *q, const void *qd,
+                   const void *qdd, void *tau, const BaseParams<T> &base, cudaStream_t s)
+{
+    const int n = m->n;
+    const size_t smem = dhp_smem_per_thread<T>(n, K, n < 8 ? 0 : 8, 2) * 32;
+    if (n < 8) return launch_dhp_k<T, 32, 32, kTrigPoly, 0, 2>(m, K, B, q, qd, qdd, tau, base, smem, s);
+    if (n <= 32) return launch_dhp_k<T, 32, 32, kTrigPoly, 8, 2>(m, K, B, q, qd, qdd, tau, base, smem, s);
+    return launch_dhp_k<T, 128, 32, kTrigPoly, 8, 2>(m, K, B, q, qd, qdd, tau, base, smem, s);
 }
 
 // ---- TMEM-state kernel (FP32, n <= 32, n % 4 == 0, aligned rows)
@@ -414,6 +455,10 @@ int dh_launch(const rd_model *m, int B, const void *q, const void *qd, const voi
                                            "n %% 4 == 0, n <= 32 and 16-byte aligned rows");
             return launch_dht(m, stored ? kfull : 0, B, q, qd, qdd, tau, base, fast, s);
         }
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (kfull == RD_DHP_AUTO_F64)
+            return launch_dhp_f64<T>(m, dhp_f64_k<T>(m), B, q, qd, qdd, tau, base, s);
     }
     if ((reg_links || stages != kStages) && (!stored || tmem || !dhp_eligible<T>(m, q, qd, qdd, tau)))
         return rd_fail(RD_ERR_ARG, "rnea_batch: register state is for the stored-state "

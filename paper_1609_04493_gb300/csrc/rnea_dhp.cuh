@@ -23,10 +23,22 @@
 
 namespace rdyn {
 
+// The 16 common-normal constants per link; for rnea_dhp_kernel with the second
+// moments of kin_wrench in place of the rotational inertia.
 template <typename T, int NMAX>
 struct DhParamConsts {
     T c[NMAX * kDhConsts];
 };
+
+// S = tr(I)/2 E - I of one link's (xx, yy, zz, xy, xz, yz)
+inline void dh_second_moments(const double I[6], double S[6])
+{
+    const double h = 0.5 * (I[0] + I[1] + I[2]);
+    for (int k = 0; k < 3; ++k) {
+        S[k] = h - I[k];
+        S[3 + k] = -I[3 + k];
+    }
+}
 
 enum DhTrig { kTrigPoly = 0, kTrigSfu = 1 };
 
@@ -131,11 +143,8 @@ rnea_dhp_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int K,
     const T *qr = q + row, *qdr = qd + row, *qddr = qdd + row;
     T *taur = tau + row;
 
-    Motion<T> x;
-    x.v = mk3(base.V0[0], base.V0[1], base.V0[2]);
-    x.w = mk3(base.V0[3], base.V0[4], base.V0[5]);
-    x.a = mk3(base.dV0[0], base.dV0[1], base.dV0[2]);
-    x.al = mk3(base.dV0[3], base.dV0[4], base.dV0[5]);
+    Kin<T> x = kin_base(base.V0, base.dV0);
+    WMat<T> W = kin_wmat(x.w, x.al);
 
     // ---- forward sweep: base -> tip
     const int nchunks = n / 4, kchunks = K / 4;
@@ -151,9 +160,10 @@ rnea_dhp_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int K,
         load_dh(sc + i * kDhConsts, L);
         T s, c;
         dh_trig<T, TRIG>(qi + L.th0, &s, &c);
-        x = dh_forward(dh_rot(L.ca, L.sa, c, s), L.b, qdi, qddi, x);
+        x = kin_forward(dh_rot(L.ca, L.sa, c, s), L.b, qdi, qddi, x, W);
+        W = kin_wmat(x.w, x.al);
         LinkState<T> ls;
-        ls.Fh = bias_wrench(L.m, L.c, L.I, x);
+        ls.Fh = kin_wrench(L.m, L.c, L.I, W, x.a);
         ls.c = c;
         ls.s = s;
         return ls;
@@ -190,7 +200,8 @@ rnea_dhp_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int K,
                 load_dh_xf(sc + i * kDhConsts, X);
                 T s, c;
                 dh_trig<T, TRIG>(cq.v[j] + X.th0, &s, &c);
-                x = dh_forward(dh_rot(X.ca, X.sa, c, s), X.b, cqd.v[j], cqdd.v[j], x);
+                x = kin_forward(dh_rot(X.ca, X.sa, c, s), X.b, cqd.v[j], cqdd.v[j], x, W);
+                W = kin_wmat(x.w, x.al);
                 put_cs<T>(stc, i - K, tid, BLOCK, c, s);
             }
         }
@@ -227,14 +238,14 @@ rnea_dhp_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int K,
             T s, c;
             get_cs<T>(stc, i - K, tid, BLOCK, c, s);
             const DhRot<T> R = dh_rot(L.ca, L.sa, c, s);
-            const Wrench<T> Fh = bias_wrench(L.m, L.c, L.I, x);
+            const Wrench<T> Fh = kin_wrench(L.m, L.c, L.I, W, x.a);
             if (i == n - 1) {
                 F.f = add3(F.f, Fh.f);
                 F.n = add3(F.n, Fh.n);
             } else {
                 F = dh_carry(Rn, bn, F, Fh);
             }
-            if (i > K) x = dh_recover(R, L.b, cqd.v[j], cqdd.v[j], x);
+            if (i > K) x = kin_recover(R, L.b, cqd.v[j], cqdd.v[j], x, W);
             Rn = R;
             bn = L.b;
             ct.v[j] = F.n.z;

@@ -323,8 +323,17 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
         return rd_rnea_dh_f32(m, B, q, qd, qdd, tau, base18, 1, block, fast,
                               reglinks ? reglinks : -1, 0, regstate, stages, s);
     }
+    if constexpr (sizeof(T) == 8) {
+        // FP64, whole 16-byte chunks, untuned: common-normal frames (rnea_dhp.cuh)
+        if (variant == RD_VARIANT_AUTO && n % 4 == 0 && !block && !reglinks && !regstate &&
+            stages == kStages && aligned16(q) && aligned16(qd) && aligned16(qdd) && aligned16(tau) &&
+            rd_rnea_dhp_f64_fits(m))
+            return rd_rnea_dh_f64(m, B, q, qd, qdd, tau, base18, 1, 0, 0, RD_DHP_AUTO_F64, 0, 0,
+                                  kStages, s);
+    }
     if (variant == RD_VARIANT_AUTO) {
         // Sweep on GB300 at B = 65536 (modes x block sizes x stored links):
+        // (FP64: ragged or unaligned rows, n > 108 and tuned calls)
         // per-link state in shared memory wins while it is small (FP32 n <= 32,
         // FP64 n <= 16); FP64 up to n = 32 keeps part of it in registers; up to
         // n = 64 the first links keep their state and the rest are re-derived;

@@ -197,4 +197,114 @@ __device__ __forceinline__ Wrench<T> dh_carry(const DhRot<T> &R, V3<T> b, const 
     return F;
 }
 
+// ---- the recursion by origin accelerations
+//
+// The same motion carried as angular velocity w, angular acceleration al and the
+// (true, not spatial) acceleration a of the link's frame origin, a = dV_v + w x V_v
+// (Luh, Walker and Paul 1980). Linear velocity then appears nowhere, and the two
+// accelerations of points of a link, of the next frame's origin and of the centre
+// of mass, are a + W r with one matrix per link
+//     W = [al] + [w][w],
+// which also gives the rotational part of the bias wrench from the second moments
+// S of the mass about the centre of mass, S = tr(I)/2 E - I:
+//     I al + w x (I w) = axial part of W S,
+//     n_x = W_zx S_xy - W_yx S_xz + (W_zz - W_yy) S_yz + W_zy S_yy - W_yz S_zz
+// and cyclically. 114 multiply-adds a link (forward 52, wrench 33, carry 25, the
+// rotation's products 4) against 130 with dh_forward and bias_wrench.
+
+template <typename T>
+struct Kin {
+    V3<T> w, al, a;
+};
+
+template <typename T>
+struct WMat {
+    T xx, yy, zz, xy, xz, yx, yz, zx, zy;
+    T dx, dy, dz;  // zz - yy, xx - zz, yy - xx
+};
+
+template <typename T>
+__device__ __forceinline__ WMat<T> kin_wmat(V3<T> w, V3<T> al)
+{
+    const T sx = w.x * w.x, sy = w.y * w.y, sz = w.z * w.z;
+    WMat<T> W;
+    W.xx = -(sy + sz);
+    W.yy = -(sx + sz);
+    W.zz = -(sx + sy);
+    W.dx = sz - sy;
+    W.dy = sx - sz;
+    W.dz = sy - sx;
+    W.xy = fma(w.x, w.y, -al.z);
+    W.yx = fma(w.x, w.y, al.z);
+    W.xz = fma(w.x, w.z, al.y);
+    W.zx = fma(w.x, w.z, -al.y);
+    W.yz = fma(w.y, w.z, -al.x);
+    W.zy = fma(w.y, w.z, al.x);
+    return W;
+}
+
+// a + W r
+template <typename T>
+__device__ __forceinline__ V3<T> kin_at(const WMat<T> &W, V3<T> r, V3<T> a)
+{
+    return V3<T>{fma(W.xx, r.x, fma(W.xy, r.y, fma(W.xz, r.z, a.x))),
+                 fma(W.yx, r.x, fma(W.yy, r.y, fma(W.yz, r.z, a.y))),
+                 fma(W.zx, r.x, fma(W.zy, r.y, fma(W.zz, r.z, a.z)))};
+}
+
+// The base's motion {V_0, dV_0} as origin acceleration.
+template <typename T>
+__device__ __forceinline__ Kin<T> kin_base(const T V0[6], const T dV0[6])
+{
+    Kin<T> x;
+    x.w = mk3(V0[3], V0[4], V0[5]);
+    x.al = mk3(dV0[3], dV0[4], dV0[5]);
+    x.a = cross_add(x.w, mk3(V0[0], V0[1], V0[2]), mk3(dV0[0], dV0[1], dV0[2]));
+    return x;
+}
+
+// Motion of link i from that of link i-1 (x, W) and back.
+template <typename T>
+__device__ __forceinline__ Kin<T> kin_forward(const DhRot<T> &R, V3<T> b, T qd, T qdd,
+                                              const Kin<T> &x, const WMat<T> &W)
+{
+    Kin<T> o;
+    o.w = dh_mulT(R, x.w);
+    o.al = dh_mulT(R, x.al);
+    o.a = dh_mulT(R, kin_at(W, b, x.a));
+    o.w.z += qd;
+    o.al.z += qdd;
+    o.al.x = fma(qd, o.w.y, o.al.x);
+    o.al.y = fma(-qd, o.w.x, o.al.y);
+    return o;
+}
+
+template <typename T>
+__device__ __forceinline__ Kin<T> kin_recover(const DhRot<T> &R, V3<T> b, T qd, T qdd,
+                                              const Kin<T> &o, WMat<T> &W)
+{
+    const V3<T> w = mk3(o.w.x, o.w.y, o.w.z - qd);
+    const V3<T> al = mk3(fma(-qd, o.w.y, o.al.x), fma(qd, o.w.x, o.al.y), o.al.z - qdd);
+    Kin<T> p;
+    p.w = dh_mul(R, w);
+    p.al = dh_mul(R, al);
+    W = kin_wmat(p.w, p.al);
+    p.a = kin_at(W, mk3(-b.x, -b.y, -b.z), dh_mul(R, o.a));
+    return p;
+}
+
+// Bias wrench about the frame origin; S: second moments (xx, yy, zz, xy, xz, yz).
+template <typename T>
+__device__ __forceinline__ Wrench<T> kin_wrench(T m, V3<T> c, const T *S, const WMat<T> &W, V3<T> a)
+{
+    Wrench<T> F;
+    F.f = scale3(m, kin_at(W, c, a));
+    const V3<T> n = {
+        fma(W.zx, S[3], fma(-W.yx, S[4], fma(W.dx, S[5], fma(W.zy, S[1], -W.yz * S[2])))),
+        fma(W.xy, S[5], fma(-W.zy, S[3], fma(W.dy, S[4], fma(W.xz, S[2], -W.zx * S[0])))),
+        fma(W.yz, S[4], fma(-W.xz, S[5], fma(W.dz, S[3], fma(W.yx, S[0], -W.xy * S[1]))))};
+    F.n = cross_add(c, F.f, n);
+    return F;
+}
+
 }  // namespace rdyn
