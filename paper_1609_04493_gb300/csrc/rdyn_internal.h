@@ -64,6 +64,8 @@ void rd_build_aba64(int n, const std::vector<double> &dh64, std::vector<double> 
 // kfull of rd_rnea_dh_f64 for the rows that AUTO sends there, where
 // rd_rnea_dhp_f64_fits says so
 constexpr int RD_DHP_AUTO_F64 = -2;
+// kfull of rd_rnea_dh_f32 for rows of any length and alignment by AUTO
+constexpr int RD_DHP_AUTO_RAGGED = -3;
 bool rd_rnea_dhp_f64_fits(const rd_model *m);
 int rd_rnea_dh_f32(const rd_model *m, int B, const void *q, const void *qd, const void *qdd,
                    void *tau, const double *base18, int stored, int block, int fast,

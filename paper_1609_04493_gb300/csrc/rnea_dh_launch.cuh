@@ -100,12 +100,12 @@ int launch_dh_mode(const rd_model *m, int block, int B, const void *q, const voi
     }
 }
 
-template <typename T, int NMAX, int BLOCK, int TRIG, int RL = 0, int STG = kStages>
+template <typename T, int NMAX, int BLOCK, int TRIG, int RL = 0, int STG = kStages, bool VEC = true>
 int launch_dhp_k(const rd_model *m, int K, int B, const void *q, const void *qd, const void *qdd,
                  void *tau, const BaseParams<T> &base, size_t smem, cudaStream_t stream)
 {
     static std::atomic<uint64_t> configured{0};
-    auto kern = rnea_dhp_kernel<T, NMAX, BLOCK, TRIG, RL, STG>;
+    auto kern = rnea_dhp_kernel<T, NMAX, BLOCK, TRIG, RL, STG, VEC>;
     const uint64_t bit = 1ull << (m->device & 63);
     if (!(configured.load() & bit)) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -238,6 +238,46 @@ void dhp_default_kr(const rd_model *m, int B, int &K, int &RL, int &stages)
     stages = (n == 24 || n == 32) ? kStages : 2;
 }
 
+// FP32 rows of any length and alignment by AUTO: every link stored up to 32 links, the
+// first four in registers, or eight for the longest chains in batches beyond two
+// waves (n = 31, B = 262144: 73 us against 79; n = 29, B = 49999: 17.9 against 15.7; n =
+// 13, B = 65536: 12.5 against 10.0: the unrolled code is fetched once a block); beyond
+// 32, dhp_default_k's K. us, joint-frame kernels with element loads / now: n = 7, B =
+// 65536: 6.5 / 5.7; n = 13: 11.1 / 10.0; n = 29, B = 49999: 25.2 / 15.7; n = 63, B = 65536:
+// 108 / 47.5; n = 99: 123 / 73.5.
+template <int TRIG>
+int launch_dhp_ragged(const rd_model *m, int B, const void *q, const void *qd, const void *qdd,
+                      void *tau, const BaseParams<float> &base, cudaStream_t s)
+{
+    const int n = m->n;
+    if (n > 32) {
+        const int K = dhp_default_k<float>(m, B);
+        return launch_dhp_k<float, 128, 32, TRIG, 0, kStages, false>(
+            m, K, B, q, qd, qdd, tau, base, dhp_smem_per_thread<float>(n, K) * 32, s);
+    }
+    int RL = n < 4 ? 0 : 4;
+    if (n >= 28) {
+        static std::atomic<int> known[64][33];
+        std::atomic<int> &slot = known[m->device & 63][n];
+        int per_sm = slot.load() - 1;
+        if (per_sm < 0) {
+            per_sm = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &per_sm, rnea_dhp_kernel<float, 32, 32, TRIG, 4, 2, false>, 32,
+                dhp_smem_per_thread<float>(n, n, 4, 2) * 32);
+            slot.store(per_sm + 1);
+        }
+        const long long sms = dh_device_attr(m->device, cudaDevAttrMultiProcessorCount, 1);
+        if (2 * (long long)per_sm * sms < (long long)(B + 31) / 32) RL = 8;
+    }
+    const size_t smem = dhp_smem_per_thread<float>(n, n, RL, 2) * 32;
+    if (RL == 0)
+        return launch_dhp_k<float, 32, 32, TRIG, 0, 2, false>(m, n, B, q, qd, qdd, tau, base, smem, s);
+    if (RL == 4)
+        return launch_dhp_k<float, 32, 32, TRIG, 4, 2, false>(m, n, B, q, qd, qdd, tau, base, smem, s);
+    return launch_dhp_k<float, 32, 32, TRIG, 8, 2, false>(m, n, B, q, qd, qdd, tau, base, smem, s);
+}
+
 // FP32, n <= 32, 32-thread blocks: the first RL of the K stored links keep
 // their state in registers (RL = 4, 8, 12 or 16; K >= RL)
 template <int TRIG>
@@ -319,19 +359,21 @@ int dhp_f64_k(const rd_model *m)
     const size_t limit = (size_t)smem_sm[d].load() / 4 - 1024;  // less the block's reserve
     const int RL = n < 8 ? 0 : 8;
     int K = n;
-    while (K >= RL && dhp_smem_per_thread<T>(n, K, RL, 2) * 32 > limit) K -= 4;
+    while (K >= RL && dhp_smem_per_thread<T>(n, K, RL, 2) * 32 > limit) K = 4 * ((K - 1) / 4);
     return K >= RL ? K : -1;
 }
 
-template <typename T>
+template <typename T, bool VEC>
 int launch_dhp_f64(const rd_model *m, int K, int B, const void *q, const void *qd,
                    const void *qdd, void *tau, const BaseParams<T> &base, cudaStream_t s)
 {
     const int n = m->n;
     const size_t smem = dhp_smem_per_thread<T>(n, K, n < 8 ? 0 : 8, 2) * 32;
-    if (n < 8) return launch_dhp_k<T, 32, 32, kTrigPoly, 0, 2>(m, K, B, q, qd, qdd, tau, base, smem, s);
-    if (n <= 32) return launch_dhp_k<T, 32, 32, kTrigPoly, 8, 2>(m, K, B, q, qd, qdd, tau, base, smem, s);
-    return launch_dhp_k<T, 128, 32, kTrigPoly, 8, 2>(m, K, B, q, qd, qdd, tau, base, smem, s);
+    if (n < 8)
+        return launch_dhp_k<T, 32, 32, kTrigPoly, 0, 2, VEC>(m, K, B, q, qd, qdd, tau, base, smem, s);
+    if (n <= 32)
+        return launch_dhp_k<T, 32, 32, kTrigPoly, 8, 2, VEC>(m, K, B, q, qd, qdd, tau, base, smem, s);
+    return launch_dhp_k<T, 128, 32, kTrigPoly, 8, 2, VEC>(m, K, B, q, qd, qdd, tau, base, smem, s);
 }
 
 // ---- TMEM-state kernel (FP32, n <= 32, n % 4 == 0, aligned rows)
@@ -457,8 +499,16 @@ int dh_launch(const rd_model *m, int B, const void *q, const void *qd, const voi
         }
     }
     if constexpr (sizeof(T) == 8) {
-        if (kfull == RD_DHP_AUTO_F64)
-            return launch_dhp_f64<T>(m, dhp_f64_k<T>(m), B, q, qd, qdd, tau, base, s);
+        if (kfull == RD_DHP_AUTO_F64) {
+            const int K = dhp_f64_k<T>(m);
+            return dhp_eligible<T>(m, q, qd, qdd, tau)
+                       ? launch_dhp_f64<T, true>(m, K, B, q, qd, qdd, tau, base, s)
+                       : launch_dhp_f64<T, false>(m, K, B, q, qd, qdd, tau, base, s);
+        }
+    } else {
+        if (kfull == RD_DHP_AUTO_RAGGED)
+            return fast ? launch_dhp_ragged<kTrigSfu>(m, B, q, qd, qdd, tau, base, s)
+                        : launch_dhp_ragged<kTrigPoly>(m, B, q, qd, qdd, tau, base, s);
     }
     if ((reg_links || stages != kStages) && (!stored || tmem || !dhp_eligible<T>(m, q, qd, qdd, tau)))
         return rd_fail(RD_ERR_ARG, "rnea_batch: register state is for the stored-state "

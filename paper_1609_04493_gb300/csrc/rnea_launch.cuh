@@ -300,9 +300,12 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     variant &= 0xfff;
     const bool dhp_rows = sizeof(T) == 4 && n % 4 == 0 && n <= 128 && aligned16(q) &&
                           aligned16(qd) && aligned16(qdd) && aligned16(tau);
+    // rows of any length and alignment, untuned, for the common-normal kernel
+    const bool untuned = (!block || block == 32) && !reglinks && !regstate && stages == kStages;
+    const bool ragged = sizeof(T) == 4 && !dhp_rows && n <= 128 && untuned;
     // the common-normal kernel of the next branch overtakes the scans sooner
     // (n = 32: 7.5 us against 9.3 at B = 4096; 6.9 against 5.0 at B = 1024)
-    if (variant == RD_VARIANT_AUTO && B <= (dhp_rows ? 2048 : 152 * 32) && n <= 128) {
+    if (variant == RD_VARIANT_AUTO && B <= (dhp_rows || ragged ? 2048 : 152 * 32) && n <= 128) {
         // Fewer instances than one warp per SM: the serial recursion leaves the
         // GPU idle, and splitting each chain over lanes (the scans of Sec. III)
         // cuts latency. Measured: n = 7, B = 1024 FP64 30 us with 8 lanes vs 43
@@ -323,17 +326,19 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
         return rd_rnea_dh_f32(m, B, q, qd, qdd, tau, base18, 1, block, fast,
                               reglinks ? reglinks : -1, 0, regstate, stages, s);
     }
-    if constexpr (sizeof(T) == 8) {
-        // FP64, whole 16-byte chunks, untuned: common-normal frames (rnea_dhp.cuh)
-        if (variant == RD_VARIANT_AUTO && n % 4 == 0 && !block && !reglinks && !regstate &&
-            stages == kStages && aligned16(q) && aligned16(qd) && aligned16(qdd) && aligned16(tau) &&
-            rd_rnea_dhp_f64_fits(m))
+    if constexpr (sizeof(T) == 4) {
+        if (variant == RD_VARIANT_AUTO && ragged)
+            return rd_rnea_dh_f32(m, B, q, qd, qdd, tau, base18, 1, 0, fast, RD_DHP_AUTO_RAGGED, 0, 0,
+                                  kStages, s);
+    } else {
+        // FP64, untuned: common-normal frames (rnea_dhp.cuh)
+        if (variant == RD_VARIANT_AUTO && untuned && rd_rnea_dhp_f64_fits(m))
             return rd_rnea_dh_f64(m, B, q, qd, qdd, tau, base18, 1, 0, 0, RD_DHP_AUTO_F64, 0, 0,
                                   kStages, s);
     }
     if (variant == RD_VARIANT_AUTO) {
         // Sweep on GB300 at B = 65536 (modes x block sizes x stored links):
-        // (FP64: ragged or unaligned rows, n > 108 and tuned calls)
+        // (now for tuned calls, FP64 also n > 108)
         // per-link state in shared memory wins while it is small (FP32 n <= 32,
         // FP64 n <= 16); FP64 up to n = 32 keeps part of it in registers; up to
         // n = 64 the first links keep their state and the rest are re-derived;
