@@ -553,6 +553,7 @@ int rd_joint_trig_df(const double *x, double *s, double *c, int count, void *str
  */
 #define RD_RNEA_KERNEL_DH_PARAM 0x206
 #define RD_RNEA_KERNEL_DH_TMEM 0x208
+#define RD_RNEA_KERNEL_WIDE 0x20a /* FP64, small batches: sixteen lanes per instance */
 #define RD_RNEA_KERNEL_DH_HOST 0x209 /* rnea_batch_host reading mapped host arrays */
 int rd_rnea_last_config(int *kernel, int *block, int *stored_links);
 /* Where the last launch of the common-normal kernel with stored state kept it:

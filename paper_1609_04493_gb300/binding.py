@@ -24,6 +24,7 @@ RD_VARIANT_SERIAL_DH_TMEM = 8
 RD_VARIANT_SERIAL_DF = 9
 RD_FLAG_HOST_COPY = 0x4000
 RD_RNEA_KERNEL_DH_HOST = 0x209
+RD_RNEA_KERNEL_WIDE = 0x20a
 
 
 RD_FLAG_FAST_TRIG = 0x1000

@@ -67,6 +67,9 @@ constexpr int RD_DHP_AUTO_F64 = -2;
 // kfull of rd_rnea_dh_f32 for rows of any length and alignment by AUTO
 constexpr int RD_DHP_AUTO_RAGGED = -3;
 bool rd_rnea_dhp_f64_fits(const rd_model *m);
+// FP64, small batches: sixteen lanes per instance (rnea_wide.cuh), any rows
+int rd_rnea_wide_f64(const rd_model *m, int B, const void *q, const void *qd, const void *qdd,
+                     void *tau, const double *base18, cudaStream_t s);
 int rd_rnea_dh_f32(const rd_model *m, int B, const void *q, const void *qd, const void *qdd,
                    void *tau, const double *base18, int stored, int block, int fast,
                    int kfull, int tmem, int reg_links, int stages, cudaStream_t s);

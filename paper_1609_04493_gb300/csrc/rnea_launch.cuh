@@ -42,6 +42,18 @@ int max_smem_optin(int device)
     return v;
 }
 
+int sm_count(int device)
+{
+    static std::atomic<int> cache[64];
+    const int d = device & 63;
+    int v = cache[d].load();
+    if (v == 0) {
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) v = 1;
+        cache[d].store(v);
+    }
+    return v;
+}
+
 // Raise a kernel's dynamic shared-memory limit once per device.
 template <typename K>
 cudaError_t allow_smem(K kern, int device, std::atomic<uint64_t> &done)
@@ -303,14 +315,32 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     // rows of any length and alignment, untuned, for the common-normal kernel
     const bool untuned = (!block || block == 32) && !reglinks && !regstate && stages == kStages;
     const bool ragged = sizeof(T) == 4 && !dhp_rows && n <= 128 && untuned;
+    if constexpr (sizeof(T) == 8) {
+        // FP64, untuned: sixteen lanes per instance (rnea_wide.cuh) while that takes
+        // fewer cycles of the FP64 unit than one thread per instance, whose time
+        // is flat up to a warp per SM; then the common-normal kernel, or beyond its
+        // 108 links the kernels below. us at B = 1024 / 6000 / 8192, sixteen lanes / one
+        // thread (lane scans below 4864 before): n = 1: 5.5 / 14.5 / 18.7 and 6.6 flat;
+        // n = 2: 6.4 / 16.9 / 22.2 and 11.2; n = 7: 10.2 / 29.4 / 39.9 and 33.1 (scans
+        // 29.5); n = 32: 32.6 / 113 / 147 and 135 (49.6); n = 64: 63.7 / 250 / 331 and
+        // 342 (75.2). n = 128: the scans lead below 4864 (4096: 465 / 502), sixteen
+        // lanes at 6000 (634 / 959).
+        const bool fits = rd_rnea_dhp_f64_fits(m);
+        const long long per_sm = n == 1 ? 12 : n <= 3 ? 22 : 44;
+        if (variant == RD_VARIANT_AUTO && untuned && (fits || B > 152 * 32) &&
+            B <= per_sm * sm_count(m->device))
+            return rd_rnea_wide_f64(m, B, q, qd, qdd, tau, base18, s);
+        if (variant == RD_VARIANT_AUTO && untuned && fits)
+            return rd_rnea_dh_f64(m, B, q, qd, qdd, tau, base18, 1, 0, 0, RD_DHP_AUTO_F64, 0, 0,
+                                  kStages, s);
+    }
     // the common-normal kernel of the next branch overtakes the scans sooner
     // (n = 32: 7.5 us against 9.3 at B = 4096; 6.9 against 5.0 at B = 1024)
     if (variant == RD_VARIANT_AUTO && B <= (dhp_rows || ragged ? 2048 : 152 * 32) && n <= 128) {
         // Fewer instances than one warp per SM: the serial recursion leaves the
         // GPU idle, and splitting each chain over lanes (the scans of Sec. III)
-        // cuts latency. Measured: n = 7, B = 1024 FP64 30 us with 8 lanes vs 43
-        // serial; n = 32, B = 1024 FP32 5.1 us with 16 lanes vs 8.4 serial;
-        // from B = 8192 on the serial form wins.
+        // cuts latency. Measured: n = 32, B = 1024 FP32 5.1 us with 16 lanes vs 8.4
+        // serial; from B = 8192 on the serial form wins.
         int lanes = 2;
         while (lanes < 16 && lanes < n) lanes <<= 1;
         while (lanes * 8 < n) lanes <<= 1;
@@ -329,11 +359,6 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     if constexpr (sizeof(T) == 4) {
         if (variant == RD_VARIANT_AUTO && ragged)
             return rd_rnea_dh_f32(m, B, q, qd, qdd, tau, base18, 1, 0, fast, RD_DHP_AUTO_RAGGED, 0, 0,
-                                  kStages, s);
-    } else {
-        // FP64, untuned: common-normal frames (rnea_dhp.cuh)
-        if (variant == RD_VARIANT_AUTO && untuned && rd_rnea_dhp_f64_fits(m))
-            return rd_rnea_dh_f64(m, B, q, qd, qdd, tau, base18, 1, 0, 0, RD_DHP_AUTO_F64, 0, 0,
                                   kStages, s);
     }
     if (variant == RD_VARIANT_AUTO) {

@@ -43,7 +43,7 @@ def run(rd, n, B, dtype, offset=0, variant=0):
     return oracle.rel_err(tau[idx], ref)
 
 
-@pytest.mark.parametrize("dtype,B", [("float32", 2049), ("float32", 40000), ("float64", 4897)])
+@pytest.mark.parametrize("dtype,B", [("float32", 2049), ("float32", 40000), ("float64", 8161)])
 @pytest.mark.parametrize("n", [1, 2, 3, 5, 6, 7, 9, 11, 30, 31, 33, 63, 65, 107, 109, 127])
 def test_ragged_lengths(cuda_lib, n, dtype, B):
     if B == 40000 and n > 33:
@@ -54,7 +54,7 @@ def test_ragged_lengths(cuda_lib, n, dtype, B):
 @pytest.mark.parametrize("dtype", ["float32", "float64"])
 @pytest.mark.parametrize("n,offset", [(4, 1), (8, 3), (32, 1), (36, 2), (7, 1), (29, 3)])
 def test_unaligned_rows(cuda_lib, n, offset, dtype):
-    assert run(cuda_lib, n, 5001, dtype, offset=offset) <= TOL[dtype]
+    assert run(cuda_lib, n, 8161, dtype, offset=offset) <= TOL[dtype]
     assert cuda_lib.rnea_last_config()[0] == cuda_lib.RD_RNEA_KERNEL_DH_PARAM
 
 
