@@ -265,8 +265,7 @@ class Model:
 
 
 def _dtype_code(t):
-    import torch
-
+    torch = _torch or _import_torch()
     if t.dtype == torch.float32:
         return RD_F32
     if t.dtype == torch.float64:
@@ -281,7 +280,48 @@ def _base_arg(base):
     return b, _dptr(b)
 
 
+_torch = None
+_raw_stream = None
+
+
+def _import_torch():
+    """torch, imported on the first call that needs it."""
+    global _torch, _raw_stream
+    import torch
+
+    # the current stream's handle without building a Stream object (2 us a call)
+    _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    _torch = torch
+    return torch
+
+
+def _stream_handle(stream, t):
+    """cudaStream_t of ``stream``, or of the current stream of t's device."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(t.get_device())
+    return _torch.cuda.current_stream(t.device).cuda_stream
+
+
 def _check_batch(model, *ts):
+    # what nearly every call passes, in few steps (the checks below took as long as a
+    # small kernel): plain contiguous CUDA tensors of one dtype and shape [B, n]
+    torch = _torch or _import_torch()
+    tensor, ref = torch.Tensor, ts[0]
+    if type(ref) is tensor:
+        shape, dtype = ref.shape, ref.dtype
+        for t in ts:
+            if (type(t) is not tensor or not t.is_cuda or t.dtype is not dtype
+                    or t.shape != shape or not t.is_contiguous()):
+                break
+        else:
+            if len(shape) == 2 and shape[1] == model.n:
+                return
+    _check_batch_verbose(model, *ts)
+
+
+def _check_batch_verbose(model, *ts):
     import torch
 
     ref = ts[0]
@@ -300,19 +340,15 @@ def _check_batch(model, *ts):
 
 def rnea(model, q, qd, qdd, out=None, base=None, variant=RD_VARIANT_AUTO, stream=None):
     """tau = ID(q, qd, qdd, V_0, dV_0, F_{n+1}) on the GPU (rnea_batch)."""
-    import torch
-
     _check_batch(model, q, qd, qdd)
     if out is None:
-        out = torch.empty_like(q)
+        out = _torch.empty_like(q)
     else:
         _check_batch(model, q, out)
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device)
     keep, bp = _base_arg(base)
-    _check(_lib.rnea_batch(model.handle, q.shape[0], _dtype_code(q), q.data_ptr(), qd.data_ptr(),
+    _check(_lib.rnea_batch(model._h, q.shape[0], _dtype_code(q), q.data_ptr(), qd.data_ptr(),
                            qdd.data_ptr(), out.data_ptr(), bp, int(variant),
-                           ctypes.c_void_p(stream.cuda_stream)))
+                           _stream_handle(stream, q)))
     del keep
     return out
 
@@ -367,10 +403,12 @@ def rnea_vjp(model, q, qd, qdd, w, base=None, mode=RD_VJP_AUTO, workspace=None, 
     In store mode (or AUTO with a workspace) the caller may pass a preallocated
     uint8 CUDA tensor as ``workspace``; for RD_VJP_STORE without one, a tensor of
     the required size is allocated here (torch's allocator), never in the library."""
-    import torch
-
     _check_batch(model, q, qd, qdd, w)
-    gq, gqd, gqdd = out if out is not None else (torch.empty_like(q) for _ in range(3))
+    torch = _torch
+    if out is not None:
+        gq, gqd, gqdd = out
+    else:
+        gq, gqd, gqdd = torch.empty_like(q), torch.empty_like(q), torch.empty_like(q)
     code = _dtype_code(q)
     ws_ptr, ws_bytes = None, 0
     if workspace is None and (mode & 0xff) == RD_VJP_STORE:
@@ -378,13 +416,11 @@ def rnea_vjp(model, q, qd, qdd, w, base=None, mode=RD_VJP_AUTO, workspace=None, 
                                 device=q.device)
     if workspace is not None:
         ws_ptr, ws_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device)
     keep, bp = _base_arg(base)
-    _check(_lib.rnea_vjp(model.handle, q.shape[0], code, q.data_ptr(), qd.data_ptr(),
+    _check(_lib.rnea_vjp(model._h, q.shape[0], code, q.data_ptr(), qd.data_ptr(),
                          qdd.data_ptr(), w.data_ptr(), gq.data_ptr(), gqd.data_ptr(),
                          gqdd.data_ptr(), bp, int(mode), ws_ptr, ws_bytes,
-                         ctypes.c_void_p(stream.cuda_stream)))
+                         _stream_handle(stream, q)))
     del keep
     return gq, gqd, gqdd
 
@@ -444,9 +480,9 @@ RD_WARN_TIMEOUT = 2
 
 def aba_workspace_bytes(model, B, dtype_code, flags=0):
     """Workspace bytes aba_batch needs for B states."""
-    lib = load()
+    lib = _lib or load()
     out = ctypes.c_size_t()
-    _check(lib.aba_workspace_size(model.handle, int(B), int(dtype_code), int(flags),
+    _check(lib.aba_workspace_size(model._h, int(B), int(dtype_code), int(flags),
                                   ctypes.byref(out)))
     return out.value
 
@@ -457,26 +493,23 @@ def aba(model, q, qd, tau, base=None, workspace=None, status=None, out=None, str
     of aba_workspace_bytes() is taken from torch's allocator when not given; pass a
     preallocated one (and ``out``) for allocation-free repeated calls. ``status``:
     optional int32 CUDA tensor [B] receiving per-instance warnings."""
-    import torch
-
     _check_batch(model, q, qd, tau)
+    torch = _torch
     qdd = out if out is not None else torch.empty_like(q)
     code = _dtype_code(q)
     if workspace is None:
         workspace = torch.empty(aba_workspace_bytes(model, q.shape[0], code, flags),
                                 dtype=torch.uint8, device=q.device)
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device)
     keep, bp = _base_arg(base)
     st_ptr = None
     if status is not None:
         if status.dtype != torch.int32 or not status.is_cuda or status.numel() < q.shape[0]:
             raise ValueError("status must be an int32 CUDA tensor with B entries")
         st_ptr = status.data_ptr()
-    _check(_lib.aba_batch(model.handle, q.shape[0], code, q.data_ptr(), qd.data_ptr(),
+    _check(_lib.aba_batch(model._h, q.shape[0], code, q.data_ptr(), qd.data_ptr(),
                           tau.data_ptr(), qdd.data_ptr(), bp, st_ptr, int(flags), workspace.data_ptr(),
                           workspace.numel() * workspace.element_size(),
-                          ctypes.c_void_p(stream.cuda_stream)))
+                          _stream_handle(stream, q)))
     del keep
     return qdd
 
@@ -608,17 +641,13 @@ def fleet_batch(plan, q, qd, in2, out=None, base=None, status=None,
 
 def jsiia(model, q, qd, tau, base=None, status=None, out=None, stream=None):
     """qdd = FD(q, qd, tau) by joint-space-inertia inversion (jsiia_batch), n <= 32."""
-    import torch
-
     _check_batch(model, q, qd, tau)
-    qdd = out if out is not None else torch.empty_like(q)
-    if stream is None:
-        stream = torch.cuda.current_stream(q.device)
+    qdd = out if out is not None else _torch.empty_like(q)
     keep, bp = _base_arg(base)
     st_ptr = status.data_ptr() if status is not None else None
-    _check(_lib.jsiia_batch(model.handle, q.shape[0], _dtype_code(q), q.data_ptr(), qd.data_ptr(),
+    _check(_lib.jsiia_batch(model._h, q.shape[0], _dtype_code(q), q.data_ptr(), qd.data_ptr(),
                             tau.data_ptr(), qdd.data_ptr(), bp, st_ptr,
-                            ctypes.c_void_p(stream.cuda_stream)))
+                            _stream_handle(stream, q)))
     del keep
     return qdd
 

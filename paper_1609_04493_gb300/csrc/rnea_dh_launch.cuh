@@ -152,6 +152,14 @@ int dh_device_attr(int device, cudaDeviceAttr attr, int fallback)
     return v;
 }
 
+int dh_sms(int device)
+{
+    static std::atomic<int> cache[64];
+    const int d = device & 63;
+    if (cache[d].load() == 0) cache[d].store(dh_device_attr(device, cudaDevAttrMultiProcessorCount, 1));
+    return cache[d].load();
+}
+
 // Default K for the parameter-constant kernel (32-thread blocks). On GB300 at
 // B = 65536 the fastest K at every length was the largest that still leaves 7
 // blocks per SM, so the batch runs in at most two waves (n = 16: K = 16, 10.8 us;
@@ -228,7 +236,7 @@ void dhp_default_kr(const rd_model *m, int B, int &K, int &RL, int &stages)
             &per_sm, rnea_dhp_kernel<float, 32, 32, TRIG, 4, 2>, 32, smem);
         slot.store(per_sm + 1);
     }
-    const long long sms = dh_device_attr(m->device, cudaDevAttrMultiProcessorCount, 1);
+    const long long sms = dh_sms(m->device);
     if ((long long)per_sm * sms >= 2 * ((long long)(B + 31) / 32)) {
         RL = 4;
         stages = 2;
@@ -267,7 +275,7 @@ int launch_dhp_ragged(const rd_model *m, int B, const void *q, const void *qd, c
                 dhp_smem_per_thread<float>(n, n, 4, 2) * 32);
             slot.store(per_sm + 1);
         }
-        const long long sms = dh_device_attr(m->device, cudaDevAttrMultiProcessorCount, 1);
+        const long long sms = dh_sms(m->device);
         if (2 * (long long)per_sm * sms < (long long)(B + 31) / 32) RL = 8;
     }
     const size_t smem = dhp_smem_per_thread<float>(n, n, RL, 2) * 32;
