@@ -105,12 +105,12 @@ enum rd_status {
  * block, exchanging their shift terms per link), three warps per 32 instances.
  * Same results to rounding; same exclusions. */
 #define RD_ABA_THREE_WARPS 0x100
-/* aba_batch flag, RD_F32 data with double-float updates: the
+/* aba_batch flag, RD_F64 data or RD_F32 data with double-float updates: the
  * articulated-inertia recursion and the solves spread over three lanes per
  * instance (one per axis; ten instances per warp), beside a warp for the bias
  * sweeps. Same exclusions. The library's choice for n >= 3 while the batch is
- * resident at once (B <= 120 per SM; 160 with double-float bias sweeps), where it
- * also serves RD_ABA_TWO_WARPS and RD_ABA_THREE_WARPS (the same split of the work,
+ * resident at once (RD_F64: B <= 60 per SM where one warp per instance does not lead;
+ * RD_F32: 120, or 160 with double-float bias sweeps), where for RD_F32 it also serves RD_ABA_TWO_WARPS and RD_ABA_THREE_WARPS (the same split of the work,
  * results to rounding). */
 #define RD_ABA_THREE_LANES 0x200
 /* aba_batch test hook, only with RD_ABA_TWO_WARPS: the articulated-inertia warp

@@ -164,6 +164,101 @@ __device__ __forceinline__ AbiT<D> aba_dh_update(const AbiT<D> &P, D c, D s, con
     return o;
 }
 
+// aba_dh_update in fewer operations, for FP64 data with one thread per instance,
+// where every FP64 instruction counts (about 165 against 190): the plane rotations
+// by x' = y + t, y' = x - t with t = c^2 (x - y) - 2 c s z; and with Bh = B_r + PT / 2 and
+// Y = [b] Bh the shift's terms of C as Y + Y^T, added up in the multiply-adds (the
+// last of them, -[b] A_r [b], is symmetric).
+template <typename D>
+__device__ __forceinline__ Sym3<D> rotz_sym_few(const Sym3<D> &S, D c, D s, D cc, D cs, D c2, D s2)
+{
+    const D d = S.xx - S.yy;
+    const D t = fma(cc, d, -s2 * S.xy);
+    return Sym3<D>{S.yy + t, S.xx - t, S.zz, fma(cs, d, c2 * S.xy), fma(c, S.xz, -s * S.yz),
+                   fma(s, S.xz, c * S.yz)};
+}
+
+template <typename D>
+__device__ __forceinline__ AbiT<D> aba_dh_update_few(const AbiT<D> &P, D c, D s, const D *r,
+                                                     const D *ri)
+{
+    const D ca = r[0], sa = r[1];
+    const D ca2 = r[25], sa2 = r[26], casa = r[27], c2a = r[28], s2a = r[29];
+    const D cc = c * c, cs = c * s, c2 = fma(-s, s, cc), s2 = cs + cs;
+    Sym3<D> A = rotz_sym_few(P.A, c, s, cc, cs, c2, s2);
+    D B2[6];  // Rz Bm Rz^T, columns 0 and 1 (column 2 of Bm is zero)
+#pragma unroll
+    for (int rr = 0; rr < 3; ++rr) {
+        D u0, u1;  // row rr of Rz Bm
+        if (rr == 0) {
+            u0 = fma(c, P.Bm[0], -s * P.Bm[3]);
+            u1 = fma(c, P.Bm[1], -s * P.Bm[4]);
+        } else if (rr == 1) {
+            u0 = fma(s, P.Bm[0], c * P.Bm[3]);
+            u1 = fma(s, P.Bm[1], c * P.Bm[4]);
+        } else {
+            u0 = P.Bm[6];
+            u1 = P.Bm[7];
+        }
+        B2[2 * rr] = fma(c, u0, -s * u1);
+        B2[2 * rr + 1] = fma(s, u0, c * u1);
+    }
+    const D dc = P.C.xx - P.C.yy, tc = fma(cc, dc, -s2 * P.C.xy);
+    const D Cxx = P.C.yy + tc, Cyy = P.C.xx - tc, Cxy = fma(cs, dc, c2 * P.C.xy);
+    // about x: A's (y, z) plane, Bm's rows 1, 2 and column 1, C's y
+    {
+        const D d = A.yy - A.zz, t = fma(ca2, d, -s2a * A.yz);
+        A = Sym3<D>{A.xx, A.zz + t, A.yy - t, fma(ca, A.xy, -sa * A.xz), fma(sa, A.xy, ca * A.xz),
+                    fma(casa, d, c2a * A.yz)};
+    }
+    D Br[9];
+    Br[0] = B2[0];
+    Br[3] = fma(ca, B2[2], -sa * B2[4]);
+    Br[6] = fma(sa, B2[2], ca * B2[4]);
+    const D col[3] = {B2[1], fma(ca, B2[3], -sa * B2[5]), fma(sa, B2[3], ca * B2[5])};
+#pragma unroll
+    for (int rr = 0; rr < 3; ++rr) {
+        Br[3 * rr + 1] = ca * col[rr];
+        Br[3 * rr + 2] = sa * col[rr];
+    }
+    // PT = ([b] A)^T: row k is b x (column k of A)
+    const D b0 = r[2], b1 = r[3], b2 = r[4];
+    const D Ac[9] = {A.xx, A.xy, A.xz, A.xy, A.yy, A.yz, A.xz, A.yz, A.zz};
+    D PT[9], H[9];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const D x = Ac[3 * k], y = Ac[3 * k + 1], z = Ac[3 * k + 2];
+        PT[3 * k] = fma(b1, z, -b2 * y);
+        PT[3 * k + 1] = fma(b2, x, -b0 * z);
+        PT[3 * k + 2] = fma(b0, y, -b1 * x);
+    }
+    const D half = D(0.5);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) H[k] = fma(half, PT[k], Br[k]);
+    const D m = ri[6], mcx = ri[16], mcy = ri[17], mcz = ri[18];
+    const D t0 = b0 + b0, t1 = b1 + b1, t2 = b2 + b2;
+    AbiT<D> o;
+    o.A = Sym3<D>{A.xx + m, A.yy + m, A.zz + m, A.xy, A.xz, A.yz};
+    o.Bm[0] = Br[0] + PT[0];
+    o.Bm[1] = Br[1] + PT[1] + mcz;
+    o.Bm[2] = Br[2] + PT[2] - mcy;
+    o.Bm[3] = Br[3] + PT[3] - mcz;
+    o.Bm[4] = Br[4] + PT[4];
+    o.Bm[5] = Br[5] + PT[5] + mcx;
+    o.Bm[6] = Br[6] + PT[6] + mcy;
+    o.Bm[7] = Br[7] + PT[7] - mcx;
+    o.Bm[8] = Br[8] + PT[8];
+    // C' = C_r + Y + Y^T + C_o, Y_0j = b1 H_2j - b2 H_1j, Y_1j = b2 H_0j - b0 H_2j,
+    // Y_2j = b0 H_1j - b1 H_0j
+    o.C.xx = fma(t1, H[6], fma(-t2, H[3], Cxx + ri[19]));
+    o.C.yy = fma(t2, H[1], fma(-t0, H[7], fma(ca2, Cyy, ri[20])));
+    o.C.zz = fma(t0, H[5], fma(-t1, H[2], fma(sa2, Cyy, ri[21])));
+    o.C.xy = fma(b1, H[7], fma(-b2, H[4], fma(b2, H[0], fma(-b0, H[6], fma(ca, Cxy, ri[22])))));
+    o.C.xz = fma(b1, H[8], fma(-b2, H[5], fma(b0, H[3], fma(-b1, H[0], fma(sa, Cxy, ri[23])))));
+    o.C.yz = fma(b2, H[2], fma(-b0, H[8], fma(b0, H[4], fma(-b1, H[1], fma(casa, Cyy, ri[24])))));
+    return o;
+}
+
 // Sweep-1 state of a link, F_hat (6) then cos, sin, in the bias precision TB:
 // for TB = T the slots 0..5, 8, 9 of the kAbaStateScalars-wide layout; for TB
 // = DF eight pairs per link, [link][8][instance], in the same workspace
@@ -274,6 +369,10 @@ __device__ __forceinline__ int aba_dh_instance(const T *sc, const D *sd, int n,
     // at one warp per scheduler every miss stalls issue. Its sweeps run one
     // link per iteration.
     constexpr bool kRolled = std::is_same<D, DF>::value;
+    // FP64 data: F and z_hat obey the same carry in the same precision and only the
+    // sum of their z moments is used, so F carries both (22 operations a link less)
+    constexpr bool kMerge = std::is_same<T, D>::value && std::is_same<Z, D>::value &&
+                            std::is_same<TB, T>::value;
     Wrench<TB> F;
     F.f = mk3(dcvt<TB>(base.Fn[0]), dcvt<TB>(base.Fn[1]), dcvt<TB>(base.Fn[2]));
     F.n = mk3(dcvt<TB>(base.Fn[3]), dcvt<TB>(base.Fn[4]), dcvt<TB>(base.Fn[5]));
@@ -318,6 +417,10 @@ __device__ __forceinline__ int aba_dh_instance(const T *sc, const D *sd, int n,
             Jh.Bm[6] = ri[17];  Jh.Bm[7] = -ri[16]; Jh.Bm[8] = zero;
             Jh.C = Sym3<D>{ri[19], ri[20], ri[21], ri[22], ri[23], ri[24]};
         } else {
+            if constexpr (kMerge) {
+                F.f = mk3(fma(Uv[0], chat, F.f.x), fma(Uv[1], chat, F.f.y), fma(Uv[2], chat, F.f.z));
+                F.n = mk3(fma(Uw[0], chat, F.n.x), fma(Uw[1], chat, F.n.y), fma(Uw[2], chat, F.n.z));
+            }
             F = dh_carry(Rn, bn, F, Fh);
             // P = J_hat_{i+1} - U U^T / Omega: its w_z row and column vanish
             AbiT<D> P;
@@ -334,10 +437,13 @@ __device__ __forceinline__ int aba_dh_instance(const T *sc, const D *sd, int n,
             }
             P.C = Sym3<D>{fma(-wx, Uw[0], Jh.C.xx), fma(-wy, Uw[1], Jh.C.yy), D(0),
                           fma(-wx, Uw[1], Jh.C.xy), D(0), D(0)};
-            Jh = aba_dh_update(P, cn, sn, sd + (i + 1) * kAbaDh64, ri);
+            if constexpr (kMerge) Jh = aba_dh_update_few(P, cn, sn, sd + (i + 1) * kAbaDh64, ri);
+            else Jh = aba_dh_update(P, cn, sn, sd + (i + 1) * kAbaDh64, ri);
             // z_hat_i = X^T (z_hat_{i+1} + U_{i+1} c_hat_{i+1})
             Wrench<Z> zz;
-            if constexpr (kZrec) {  // one fused multiply-add per component
+            if constexpr (kMerge) {
+                zz = z;
+            } else if constexpr (kZrec) {  // one fused multiply-add per component
                 zz.f = mk3(fma(Uv[0], chat, z.f.x), fma(Uv[1], chat, z.f.y),
                            fma(Uv[2], chat, z.f.z));
                 zz.n = mk3(fma(Uw[0], chat, z.n.x), fma(Uw[1], chat, z.n.y),
@@ -350,8 +456,10 @@ __device__ __forceinline__ int aba_dh_instance(const T *sc, const D *sd, int n,
             }
             // z_hat_i = Ad^T zz: the carry of spatial_dh.cuh without a wrench to add
             // (adding zeros is not an identity in IEEE arithmetic, so it would run)
-            z.f = dh_mul(RnZ, zz.f);
-            z.n = cross_add(bnZ, z.f, dh_mul(RnZ, zz.n));
+            if constexpr (!kMerge) {
+                z.f = dh_mul(RnZ, zz.f);
+                z.n = cross_add(bnZ, z.f, dh_mul(RnZ, zz.n));
+            }
         }
         D tau_hat;
         if constexpr (kExt) tau_hat = dcvt<D>(DF(tau_i) - F.n.z);
@@ -361,7 +469,8 @@ __device__ __forceinline__ int aba_dh_instance(const T *sc, const D *sd, int n,
         const D Om = Jh.C.zz;
         if (!dpositive(Om)) bad = 1;
         invOm = drecip(Om);
-        chat = (tau_hat - dcvt<D>(z.n.z)) * invOm;
+        if constexpr (kMerge) chat = tau_hat * invOm;
+        else chat = (tau_hat - dcvt<D>(z.n.z)) * invOm;
         const Z vals[8] = {dcvt<Z>(Uv[0]), dcvt<Z>(Uv[1]), dcvt<Z>(Uv[2]), dcvt<Z>(Uw[0]),
                            dcvt<Z>(Uw[1]), dcvt<Z>(Uw[2]), dcvt<Z>(chat), dcvt<Z>(invOm)};
 #pragma unroll
@@ -378,7 +487,8 @@ __device__ __forceinline__ int aba_dh_instance(const T *sc, const D *sd, int n,
         }
         cn = dcvt<D>(c);
         sn = dcvt<D>(s);
-        if constexpr (kZrec) {
+        if constexpr (kMerge) {
+        } else if constexpr (kZrec) {
             RnZ = dh_rot(ri[0], ri[1], cn, sn);
             bnZ = mk3(ri[2], ri[3], ri[4]);
         } else {

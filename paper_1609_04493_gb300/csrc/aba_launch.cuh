@@ -233,6 +233,33 @@ bool aba_use_tri(int n, int B, int flags, bool ext)
     return !ext && B <= 2048;
 }
 
+inline int aba_sms(int device)
+{
+    static std::atomic<int> cache[64];
+    std::atomic<int> &slot = cache[device & 63];
+    int v = slot.load();
+    if (!v) {
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
+        slot.store(v);
+    }
+    return v;
+}
+
+// FP64 data: the FP64 unit does about 150 instructions a link for ten instances
+// instead of 415 for 32, so three lanes lead while two blocks of thirty per SM hold
+// the batch and one warp per instance (n >= 48, B <= 512) does not. us, one thread / three
+// lanes: n = 7: 78 / 49.5 up to B = 4096, 78 / 68 at 8192, 85 / 97 at 12000; n = 16: 179 /
+// 111, 179 / 158, 200 / 230; n = 64: 731 / 452, 733 / 644, 826 / 944 (one warp at B = 512:
+// 366); n = 128: 1487 / 897.
+inline bool aba_use_trio_f64(const rd_model *m, int B, int flags)
+{
+    if (flags & RD_ABA_THREE_LANES) return true;
+    if (flags & (RD_ABA_THREAD_PER_INSTANCE | RD_ABA_WARP_PER_INSTANCE | RD_ABA_TWO_WARPS |
+                 RD_ABA_THREE_WARPS | RD_ABA_JOINT_FRAMES))
+        return false;
+    return m->n >= 3 && !aba_use_warp<double>(m->n, B, flags) && (long long)B <= 60LL * aba_sms(m->device);
+}
+
 // Three lanes per instance (aba_trio.cuh): by flag, else for FP32 data with
 // double-float updates (also where the two- or three-warp form is asked for, which
 // it supersedes there) while the batch is resident at once, which is what the
@@ -249,15 +276,7 @@ inline bool aba_use_trio(const rd_model *m, int B, int flags, bool ext)
     if (flags & (RD_ABA_THREAD_PER_INSTANCE | RD_ABA_WARP_PER_INSTANCE | RD_ABA_JOINT_FRAMES |
                  RD_ABA_SCANS_IN_DTYPE | RD_ABA_FP64_UPDATE | RD_ABA_TEST_WITHHOLD))
         return false;
-    static std::atomic<int> sms[64];
-    std::atomic<int> &slot = sms[m->device & 63];
-    int count = slot.load();
-    if (!count) {
-        if (cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, m->device) != cudaSuccess)
-            return false;
-        slot.store(count);
-    }
-    return m->n >= 3 && (long long)B <= (ext ? 160LL : 120LL) * count;
+    return m->n >= 3 && (long long)B <= (ext ? 160LL : 120LL) * aba_sms(m->device);
 }
 
 template <typename T>
@@ -284,8 +303,8 @@ int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const 
                                        "RD_ABA_THREE_WARPS, RD_ABA_THREE_LANES and "
                                        "RD_ABA_THREAD_PER_INSTANCE exclude one another, and the "
                                        "first four RD_ABA_JOINT_FRAMES and RD_ABA_SCANS_IN_DTYPE");
-        if ((flags & RD_ABA_THREE_LANES) && (sizeof(T) != 4 || (flags & RD_ABA_FP64_UPDATE)))
-            return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_THREE_LANES takes RD_F32 data with "
+        if ((flags & RD_ABA_THREE_LANES) && sizeof(T) == 4 && (flags & RD_ABA_FP64_UPDATE))
+            return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_THREE_LANES takes RD_F64 data, or RD_F32 data with "
                                        "double-float updates");
     }
     const bool withhold = (flags & RD_ABA_TEST_WITHHOLD) != 0;
@@ -294,6 +313,9 @@ int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const 
     if constexpr (sizeof(T) == 4) {
         if (aba_use_trio(m, B, flags, ext))
             return rd_aba_trio_f32(m, B, q, qd, tau, qdd, status, ws, base18, ext, s);
+    } else {
+        if (aba_use_trio_f64(m, B, flags))
+            return rd_aba_trio_f64(m, B, q, qd, tau, qdd, status, ws, base18, s);
     }
     if (aba_use_tri<T>(m->n, B, flags, ext)) {
         if constexpr (sizeof(T) == 4)

@@ -133,6 +133,8 @@ int rd_aba_tri_f64(const rd_model *m, int B, const void *q, const void *qd, cons
 int rd_aba_trio_f32(const rd_model *m, int B, const void *q, const void *qd, const void *tau,
                     void *qdd, int *status, void *ws, const double *base18, bool extended_bias,
                     cudaStream_t s);
+int rd_aba_trio_f64(const rd_model *m, int B, const void *q, const void *qd, const void *tau,
+                    void *qdd, int *status, void *ws, const double *base18, cudaStream_t s);
 size_t rd_aba_ws_bytes_f32(int n, int B, int flags);
 size_t rd_aba_ws_bytes_f64(int n, int B, int flags);
 int rd_build_chain(int n, const double *M, const double *S, const double *inertia,

@@ -96,6 +96,21 @@ def test_trio_rejects_what_it_does_not_take(cuda_lib):
                   rd.RD_ABA_JOINT_FRAMES, rd.RD_ABA_SCANS_IN_DTYPE):
         with pytest.raises(rd.RdError):
             rd.aba(model, x, x, x, flags=rd.RD_ABA_THREE_LANES | other)
-    with pytest.raises(rd.RdError):
-        rd.aba(model, x.double(), x.double(), x.double(), flags=rd.RD_ABA_THREE_LANES)
     assert rd.aba(model, x[:0], x[:0], x[:0], flags=rd.RD_ABA_THREE_LANES).numel() == 0
+
+
+@pytest.mark.parametrize("B", [1, 29, 31])
+@pytest.mark.parametrize("n", [1, 3, 7, 64, 128])
+def test_trio_fp64_matches_oracle(cuda_lib, n, B):
+    """FP64 data: the bars of test_aba_gpu.py (1e-8) with a moving base."""
+    import torch
+
+    rd = cuda_lib
+    ch = chaingen.make_chain(n, seed=chaingen.BASE_SEED + 9 * n)
+    st = chaingen.make_states(B, n, seed=73, kinds=("q", "qd", "tau"))
+    x = [torch.from_numpy(st[k]).cuda() for k in ("q", "qd", "tau")]
+    ref = oracle.fd_aba(ch, *(st[k] for k in ("q", "qd", "tau")), base=BASE)
+    trio = rd.aba(rd.Model(ch), *x, base=BASE, flags=rd.RD_ABA_THREE_LANES)
+    one = rd.aba(rd.Model(ch), *x, base=BASE, flags=rd.RD_ABA_THREAD_PER_INSTANCE)
+    assert oracle.rel_err(trio.cpu().numpy(), ref) <= 1e-8
+    assert oracle.rel_err(one.cpu().numpy(), ref) <= 1e-8
