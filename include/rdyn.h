@@ -280,7 +280,8 @@ int rnea_batch_host(rd_model *model, int B, int dtype, const void *q, const void
 /* Modes of rnea_vjp (OR-able with RD_FLAG_FAST_TRIG and RD_VJP_FLAG_JOINT_FRAMES).
  * Rows with n % 4 == 0, n <= 128 and 16-byte aligned arrays run in the
  * common-normal link frames of RD_VARIANT_SERIAL_DH, with the link constants as
- * a kernel parameter; other rows in the joint frames. */
+ * a kernel parameter; other rows too, or in the joint frames where that is faster
+ * (short FP32 chains). */
 enum rd_vjp_mode {
     RD_VJP_AUTO = 0,      /* library's choice (FP64 with a large enough workspace: store) */
     RD_VJP_STORE = 1,     /* keep the forward sweep's state in the workspace */

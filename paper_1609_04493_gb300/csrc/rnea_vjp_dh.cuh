@@ -39,7 +39,28 @@ __device__ __forceinline__ void fb_backward_dh(const DhRot<T> &R, V3<T> b, T w, 
     fw = pw;
 }
 
-template <typename T, int NMAX, int BLOCK, int MODE, int TRIG>
+// The aligned pieces of chunk c of a row (ragged_row), read no further than the row's
+// end.
+template <typename T>
+__device__ __forceinline__ Chunk<T> ld_pieces(const RaggedRow<T> &row, int n, int c)
+{
+    Chunk<T> v;
+    const int left = row.off + n - 4 * c;
+    const T *p = row.p + 4 * c;
+    if (left >= 4) {
+        ld_row_chunk(p, 0, v);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v.v[j] = j < left ? __ldg(p + j) : T(0);
+    }
+    return v;
+}
+
+// VEC: n % 4 == 0 and 16-byte aligned rows; without it rows of any length and
+// alignment, each array streamed in aligned 16-byte pieces and shifted in registers
+// (rnea_dhp.cuh), the gradients stored by the warp together through shared memory,
+// eight rows' 16 bytes an instruction, and the last, shorter chunk as code of its own.
+template <typename T, int NMAX, int BLOCK, int MODE, int TRIG, bool VEC = true>
 __global__ void __launch_bounds__(BLOCK)
 rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int B,
                    const T *__restrict__ q, const T *__restrict__ qd, const T *__restrict__ qdd,
@@ -51,22 +72,28 @@ rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int
     extern __shared__ __align__(16) unsigned char vjp_smem[];
     T *sst = reinterpret_cast<T *>(vjp_smem);
     constexpr bool kStored = MODE == kVjpStore || MODE == kVjpStoreShared;
+    // the instance; ragged rows: lanes beyond the batch repeat the last one's work (and
+    // write its state again, the same values)
+    const int b = blockIdx.x * BLOCK + threadIdx.x;
+    const int bw = VEC || b < B ? b : B - 1;
     auto st_put = [&](int i, int k, T v) {
         if constexpr (MODE == kVjpStoreShared)
             sst[((size_t)i * kVjpStateScalars + k) * BLOCK + threadIdx.x] = v;
         else
-            ws_put(ws, B, blockIdx.x * BLOCK + threadIdx.x, i, k, v);
+            ws_put(ws, B, bw, i, k, v);
     };
     auto st_get = [&](int i, int k) -> T {
         if constexpr (MODE == kVjpStoreShared)
             return sst[((size_t)i * kVjpStateScalars + k) * BLOCK + threadIdx.x];
         else
-            return ws_get(ws, B, blockIdx.x * BLOCK + threadIdx.x, i, k);
+            return ws_get(ws, B, bw, i, k);
     };
-    const int b = blockIdx.x * BLOCK + threadIdx.x;
-    if (b >= B) return;
-    const size_t row = (size_t)b * (size_t)n;
+    if (VEC && b >= B) return;  // ragged rows: every lane stores for others
+    const size_t row = (size_t)bw * (size_t)n;
     const T *qr = q + row, *qdr = qd + row, *qddr = qdd + row, *wr = wv + row;
+    const RaggedRow<T> rr[4] = {ragged_row(qr), ragged_row(qdr), ragged_row(qddr), ragged_row(wr)};
+    Chunk<T> plo[4], phi[4], pnx[4];  // ragged rows: pieces of neighbouring chunks
+    __shared__ __align__(16) T stage[VEC ? 1 : BLOCK / 32][3][VEC ? 1 : 128];
 
     Motion<T> x;
     x.v = mk3(base.V0[0], base.V0[1], base.V0[2]);
@@ -76,15 +103,35 @@ rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int
     V3<T> fbv = mk3(T(0), T(0), T(0)), fbw = mk3(T(0), T(0), T(0));
 
     // ---- sweep 1: base -> tip
-    const int nchunks = n / 4;
+    const int nchunks = VEC ? n / 4 : (n + 3) / 4, nfull = n / 4;
     Chunk<T> cq, cqd, cqdd, cw, nq = {}, nqd = {}, nqdd = {}, nw = {};
-    ld_row_chunk(qr, 0, cq);
-    ld_row_chunk(qdr, 0, cqd);
-    ld_row_chunk(qddr, 0, cqdd);
-    ld_row_chunk(wr, 0, cw);
-    for (int kc = 0; kc < nchunks; ++kc) {
+    if constexpr (VEC) {
+        ld_row_chunk(qr, 0, cq);
+        ld_row_chunk(qdr, 0, cqd);
+        ld_row_chunk(qddr, 0, cqdd);
+        ld_row_chunk(wr, 0, cw);
+    } else {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            plo[a] = ld_pieces(rr[a], n, 0);
+            phi[a] = ld_pieces(rr[a], n, 1);
+        }
+    }
+    // ragged: the chunk's values from its pieces and the next chunk's
+    auto window = [&]() {
+        cq = shift_pieces(plo[0], phi[0], rr[0].off);
+        cqd = shift_pieces(plo[1], phi[1], rr[1].off);
+        cqdd = shift_pieces(plo[2], phi[2], rr[2].off);
+        cw = shift_pieces(plo[3], phi[3], rr[3].off);
+    };
+    auto forward_chunk = [&](int kc, auto full) {
+        constexpr bool FULL = decltype(full)::value;
         const int i0 = 4 * kc;
-        if (kc + 1 < nchunks) {
+        if constexpr (!VEC) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a) pnx[a] = ld_pieces(rr[a], n, kc + 2);
+            window();
+        } else if (kc + 1 < nchunks) {
             ld_row_chunk(qr, i0 + 4, nq);
             ld_row_chunk(qdr, i0 + 4, nqd);
             ld_row_chunk(qddr, i0 + 4, nqdd);
@@ -93,6 +140,7 @@ rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int i = i0 + j;
+            if (!FULL && i >= n) break;
             DhXf<T> X;
             load_dh_xf(sc + i * kDhConsts, X);
             T s, c;
@@ -109,11 +157,21 @@ rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int
                 for (int k = 0; k < kVjpStateScalars; ++k) st_put(i, k, vals[k]);
             }
         }
-        cq = nq;
-        cqd = nqd;
-        cqdd = nqdd;
-        cw = nw;
-    }
+        if constexpr (VEC) {
+            cq = nq;
+            cqd = nqd;
+            cqdd = nqdd;
+            cw = nw;
+        } else {
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                plo[a] = phi[a];
+                phi[a] = pnx[a];
+            }
+        }
+    };
+    for (int kc = 0; kc < nfull; ++kc) forward_chunk(kc, std::true_type());
+    if (!VEC && nfull < nchunks) forward_chunk(nfull, std::false_type());
 
     // ---- sweep 2: tip -> base
     Wrench<T> F;
@@ -124,14 +182,29 @@ rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int
     V3<T> bn = mk3(T(0), T(0), T(0));
     T qdn = T(0);
     const int last0 = n - 4;
-    ld_row_chunk(qdr, last0, cqd);
-    if constexpr (MODE == kVjpRecompute) {
-        ld_row_chunk(qr, last0, cq);
-        ld_row_chunk(qddr, last0, cqdd);
-        ld_row_chunk(wr, last0, cw);
+    if constexpr (!VEC) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            plo[a] = ld_pieces(rr[a], n, nchunks - 1);
+            phi[a] = ld_pieces(rr[a], n, nchunks);
+        }
+    } else {
+        ld_row_chunk(qdr, last0, cqd);
+        if constexpr (MODE == kVjpRecompute) {
+            ld_row_chunk(qr, last0, cq);
+            ld_row_chunk(qddr, last0, cqdd);
+            ld_row_chunk(wr, last0, cw);
+        }
     }
-    for (int i0 = last0; i0 >= 0; i0 -= 4) {
-        if (i0 > 0) {
+    auto backward_chunk = [&](int i0, auto full) {
+        constexpr bool FULL = decltype(full)::value;
+        if constexpr (!VEC) {
+            if (i0 > 0) {
+#pragma unroll
+                for (int a = 0; a < 4; ++a) pnx[a] = ld_pieces(rr[a], n, i0 / 4 - 1);
+            }
+            window();
+        } else if (i0 > 0) {
             ld_row_chunk(qdr, i0 - 4, nqd);
             if constexpr (MODE == kVjpRecompute) {
                 ld_row_chunk(qr, i0 - 4, nq);
@@ -139,10 +212,11 @@ rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int
                 ld_row_chunk(wr, i0 - 4, nw);
             }
         }
-        Chunk<T> oq, oqd, oqdd;
+        Chunk<T> oq = {}, oqd = {}, oqdd = {};
 #pragma unroll
         for (int j = 3; j >= 0; --j) {
             const int i = i0 + j;
+            if (!FULL && i >= n) continue;
             DhLink<T> L;
             load_dh(sc + i * kDhConsts, L);
             T s, c;
@@ -204,16 +278,52 @@ rnea_vjp_dh_kernel(const __grid_constant__ DhParamConsts<T, NMAX> pc, int n, int
             bn = L.b;
             qdn = cqd.v[j];
         }
-        st_chunk<T, true>(gq + row, i0, n, oq);
-        st_chunk<T, true>(gqd + row, i0, n, oqd);
-        st_chunk<T, true>(gqdd + row, i0, n, oqdd);
-        cqd = nqd;
-        if constexpr (MODE == kVjpRecompute) {
-            cq = nq;
-            cqdd = nqdd;
-            cw = nw;
+        if constexpr (VEC) {
+            st_chunk<T, true>(gq + row, i0, n, oq);
+            st_chunk<T, true>(gqd + row, i0, n, oqd);
+            st_chunk<T, true>(gqdd + row, i0, n, oqdd);
+            cqd = nqd;
+            if constexpr (MODE == kVjpRecompute) {
+                cq = nq;
+                cqdd = nqdd;
+                cw = nw;
+            }
+        } else {
+            const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+            __syncwarp();  // the chunk before has left
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                stage[wp][0][4 * lane + j] = oq.v[j];
+                stage[wp][1][4 * lane + j] = oqd.v[j];
+                stage[wp][2][4 * lane + j] = oqdd.v[j];
+            }
+            __syncwarp();
+            const int e = lane & 3;
+            const int b0 = blockIdx.x * BLOCK + 32 * wp + (lane >> 2);
+            if (i0 + e < n) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (b0 + 8 * j < B) {
+                        const size_t o = (size_t)(b0 + 8 * j) * (size_t)n + i0 + e;
+                        gq[o] = stage[wp][0][lane + 32 * j];
+                        gqd[o] = stage[wp][1][lane + 32 * j];
+                        gqdd[o] = stage[wp][2][lane + 32 * j];
+                    }
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                phi[a] = plo[a];
+                plo[a] = pnx[a];
+            }
         }
+    };
+    int top = 4 * (nchunks - 1);
+    if (!VEC && nfull < nchunks) {
+        backward_chunk(top, std::false_type());
+        top -= 4;
     }
+    for (int i0 = top; i0 >= 0; i0 -= 4) backward_chunk(i0, std::true_type());
 }
 
 }  // namespace rdyn

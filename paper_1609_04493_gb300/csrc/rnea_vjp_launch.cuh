@@ -77,7 +77,7 @@ int launch_vjp_mode(const rd_model *m, int B, const void *q, const void *qd, con
                : launch_vjp_k<T, 64, MODE, false, false>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
 }
 
-template <typename T, int NMAX, int BLOCK, int MODE, int TRIG>
+template <typename T, int NMAX, int BLOCK, int MODE, int TRIG, bool VEC = true>
 int launch_vjp_dh_k(const rd_model *m, int B, const void *q, const void *qd, const void *qdd,
                     const void *w, void *gq, void *gqd, void *gqdd, void *ws,
                     const double *base18, cudaStream_t stream)
@@ -100,14 +100,14 @@ int launch_vjp_dh_k(const rd_model *m, int B, const void *q, const void *qd, con
         smem = (size_t)m->n * kVjpStateScalars * BLOCK * sizeof(T);
         const uint64_t bit = 1ull << (m->device & 63);
         if (smem > 48 * 1024 && !(configured.load() & bit)) {
-            cudaError_t e = cudaFuncSetAttribute(rnea_vjp_dh_kernel<T, NMAX, BLOCK, MODE, TRIG>,
+            cudaError_t e = cudaFuncSetAttribute(rnea_vjp_dh_kernel<T, NMAX, BLOCK, MODE, TRIG, VEC>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  vjp_max_smem(m->device));
             if (e != cudaSuccess) return rd_cuda_fail(e, "cudaFuncSetAttribute");
             configured.fetch_or(bit);
         }
     }
-    rnea_vjp_dh_kernel<T, NMAX, BLOCK, MODE, TRIG><<<grid, BLOCK, smem, stream>>>(
+    rnea_vjp_dh_kernel<T, NMAX, BLOCK, MODE, TRIG, VEC><<<grid, BLOCK, smem, stream>>>(
         pc, m->n, B, static_cast<const T *>(q), static_cast<const T *>(qd),
         static_cast<const T *>(qdd), static_cast<const T *>(w), static_cast<T *>(gq),
         static_cast<T *>(gqd), static_cast<T *>(gqdd), static_cast<T *>(ws), bp);
@@ -238,6 +238,18 @@ int launch_vjp_dh(const rd_model *m, int B, const void *q, const void *qd, const
                  : launch_vjp_dh_k<T, 128, 64, MODE, TRIG>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
 }
 
+// Rows of any length and alignment: the common-normal kernel, re-deriving the state or
+// (MODE) in the workspace.
+template <typename T, int MODE, int TRIG>
+int launch_vjp_ragged(const rd_model *m, int B, const void *q, const void *qd, const void *qdd,
+                      const void *w, void *gq, void *gqd, void *gqdd, void *ws,
+                      const double *base18, cudaStream_t s)
+{
+    if (m->n <= 32)
+        return launch_vjp_dh_k<T, 32, 32, MODE, TRIG, false>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
+    return launch_vjp_dh_k<T, 128, 32, MODE, TRIG, false>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
+}
+
 // Common-normal kernel for whole 16-byte chunks (n % 4 == 0, n <= 128, aligned
 // rows), unless the joint-frame kernel is asked for; else the joint-frame kernel.
 template <typename T, int MODE>
@@ -262,6 +274,18 @@ int launch_vjp_any(const rd_model *m, int B, const void *q, const void *qd, cons
                                                     split, lanes, s);
         return launch_vjp_dh<T, MODE, kTrigPoly>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18,
                                                  split, lanes, s);
+    }
+    // Rows of other lengths and alignments: the common-normal kernel for FP64 (fewer FP64
+    // instructions: n = 7, B = 8192: 98 us against 107; 29: 403 against 455) and, in FP32,
+    // where its arithmetic outweighs the shifts of its loads (joint frames / this, B =
+    // 8192 and 65536: n = 7: 7.7 / 8.9, 13.3 / 16.1; 14: 12.4 / 12.0, 26.0 / 28.3; 19: 17.6
+    // / 14.2, 36.2 / 37.3; 21: 19.1 / 14.7, 40.8 / 39.8; 25: 21.8 / 16.3, 49.0 / 43.2; 63 at
+    // 65536: 139 / 104).
+    const bool pays = sizeof(T) == 8 || m->n >= 21 || (m->n >= 14 && B <= 152 * 128);
+    if (!joint_frames && pays && m->n <= 128 && split <= 0) {
+        if (sizeof(T) == 4 && fast)
+            return launch_vjp_ragged<T, MODE, kTrigSfu>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
+        return launch_vjp_ragged<T, MODE, kTrigPoly>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
     }
     return launch_vjp_mode<T, MODE>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, fast, s);
 }
