@@ -265,9 +265,9 @@ inline bool aba_use_trio_f64(const rd_model *m, int B, int flags)
 // it supersedes there) while the batch is resident at once, which is what the
 // split is for: four blocks per SM (thirty instances each, or twenty with the
 // double-float bias sweeps, where two such waves still win). Times in us on
-// GB300, the mapping taken otherwise / three lanes: n = 7: 17.6 / 14.9 at B = 1024, 34.9 / 23.7 at
-// 18240, 35.7 / 38.1 at 24000; n = 64: 346 / 218 at 18240, 360 / 355 at 24000, 352 /
-// 440 at 32768; n = 100: 822 / 708 at 16384, 990 / 852 at 24000, 938 / 1197 at
+// GB300, the mapping taken otherwise / three lanes: n = 7: 17.6 / 13.2 at B = 1024, 34.9 / 23.7 at
+// 18240, 35.7 / 38.1 at 24000; n = 64: 346 / 217 at 18240, 360 / 355 at 24000, 352 /
+// 440 at 32768; n = 100: 822 / 704 at 16384, 990 / 852 at 24000, 938 / 1197 at
 // 32768. Below three links nothing is left to split (n = 2: 5.2 / 5.3 at B = 64,
 // 7.5 / 8.0 at 16384).
 inline bool aba_use_trio(const rd_model *m, int B, int flags, bool ext)

@@ -37,9 +37,9 @@
 // instance and 2.2 k straight-line instructions a link). Splitting by axis costs
 // half as many instructions again per instance, but three times as many warps
 // run half the code each. us, GB300, FP32 data, two or three warps per 32
-// instances before / now: n = 7: B = 1024 17.6 / 14.9, 16384 28.8 / 25.5; n = 64:
-// B = 64 160 / 117, 1024 164 / 119, 4096 233 / 112, 16384 286 / 232; n = 100
-// (double-float bias): B = 64 321 / 224, 4096 516 / 293, 16384 822 / 708. The
+// instances before / now: n = 7: B = 1024 17.6 / 13.2, 16384 28.8 / 23.7; n = 64:
+// B = 64 160 / 108, 1024 164 / 110, 4096 233 / 110, 16384 286 / 216; n = 100
+// (double-float bias): B = 64 321 / 224, 4096 516 / 291, 16384 822 / 704. The
 // records are staged in shared memory (n = 64, B = 4096: 112 against 144 us from
 // global memory), the solves' inputs through a ring (112 against 126 with a ring
 // of two links).
@@ -710,6 +710,13 @@ aba_trio_kernel(const T *__restrict__ sc, const D *__restrict__ sd, int n, int B
         __syncthreads();
         return;
     }
+    // A warp without an instance (in the batch's last block) leaves: repeating the last
+    // instance's work beside the warp that has it held the block up (n = 64, B =
+    // 16384: 232 us against 216).
+    if (warp * kTrioPerWarp >= nb) {
+        __syncthreads();
+        return;
+    }
     TrioLane L = trio_lane(lane);
     int b = warp * kTrioPerWarp + L.base / 3;
     if (b >= nb) {  // beyond the batch: the last instance's work, no output
@@ -746,6 +753,10 @@ aba_trio_ext_kernel(const float *__restrict__ sc, const DF *__restrict__ sdf, in
     const int b0 = blockIdx.x * kTrioExtInstances;
     const int nb = B - b0 < kTrioExtInstances ? B - b0 : kTrioExtInstances;
     trio_block_ws(ws, wsz, n, b0, aba_bias_ws_scalars<float, DF>());
+    if (pair * kTrioPerWarp >= nb) {
+        __syncthreads();
+        return;
+    }
     TrioLane L = trio_lane(threadIdx.x & 31);
     int b = pair * kTrioPerWarp + L.base / 3;
     if (b >= nb) {
