@@ -62,6 +62,18 @@ def dh_param_flops(n, K):
     return total
 
 
+def origin_param_flops(n, K):
+    """As dh_param_flops for the recursion by origin accelerations, which the
+    parameter-constant kernel runs: a stored link costs sin/cos 26 + rotation products 4
+    + forward step 63 (three rotated vectors 39, the next origin's acceleration 18, joint
+    terms 6) + the matrix W 21 + bias wrench 60 + backward carry 44 + products 4; the
+    re-derivation of a link's motion costs 84."""
+    total = K * 222 + (n - K) * 306 - 38
+    if K < n:
+        total -= 84
+    return total
+
+
 # adjoint arithmetic per link of the common-normal kernel the bench runs (FMA = 2):
 # sweep 1 155 (sin/cos 26, rotation products 4, motion step 86, wrench-adjoint
 # step 39); sweep 2 466 (products 4, bias wrench 93, carry 44, three inertia
@@ -708,7 +720,7 @@ def run_ours(args):
     # roofline of the dominant kernel (one FP32 RNEA launch per step)
     if kern_id == rd.RD_RNEA_KERNEL_DH_PARAM:
         kname = f"rnea_dhp_kernel<float,{kern_block}>,K={kern_stored},R={kern_reg},S={kern_ring}"
-        exec_fpl = dh_param_flops(N_LINKS, kern_stored) / N_LINKS
+        exec_fpl = origin_param_flops(N_LINKS, kern_stored) / N_LINKS
     else:
         kname = f"rnea family {kern_id:#x},{kern_block}"
         exec_fpl = JOINT_FRAME_FLOP_PER_LINK

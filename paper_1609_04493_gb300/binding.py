@@ -657,9 +657,9 @@ def forward_dynamics(model, q, qd, tau, method="auto", base=None, status=None, w
     """qdd = FD(q, qd, tau) by the articulated-body algorithm (aba_batch) or the
     joint-space-inertia solve (jsiia_batch). ``auto`` takes the articulated-body
     algorithm, which on GB300 leads at every size measured once small batches
-    run with three warps per 32 instances (FP32, µs, JSIIA / ABA: n = 8, B = 256:
-    30.3 / 19.8; n = 16: 62.2 / 39.0; n = 32, B = 32 / 256 / 1024: 108 / 78.5,
-    108.5 / 78.8, 162 / 79.8; larger batches and FP64: ABA by a wider margin).
+    run with three lanes per instance (FP32, µs, JSIIA / ABA: n = 8, B = 256:
+    30.5 / 15.1; n = 16: 62.8 / 28.5; n = 32, B = 32 / 256 / 1024: 108.5 / 55.2,
+    108.7 / 55.4, 163 / 56.4; larger batches and FP64: ABA by a wider margin).
     ``jsiia`` stays available (n <= 32)."""
     if method == "auto":
         method = "aba"

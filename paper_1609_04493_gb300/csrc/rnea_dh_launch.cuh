@@ -353,7 +353,7 @@ int launch_dhp(const rd_model *m, int block, int K, int B, const void *q, const 
 // first eight links' state in registers (RL = 8) and a ring of two chunks; -1 where
 // not even the cosines and sines fit (n > 108). One warp per scheduler keeps the FP64
 // unit as busy as it gets (one DFMA a warp takes 64 cycles alone and 76 beside
-// three others, whatever the dependences), so what counts is the instructions: 122 a
+// three others, whatever the dependences), so what counts is the instructions (counted in the source): 122 a
 // stored link, 178 a re-derived one, where the joint-frame kernels took 176 and more.
 // us, joint frames / now: B = 65536: n = 8: 190 / 139, 16: 380 / 282, 32: 783 / 609,
 // 48: 1457 / 1058, 64: 2022 / 1545; B = 16384: n = 100: 901 / 650.

@@ -11,8 +11,9 @@
 //   2. base to tip, lane = component of v, w, a, al (Eq. id-forward): 7 a link;
 //   3. lane = link: the bias wrench F_hat_i (51 for 16 links);
 //   4. tip to base, lane = component of f, n (Eq. id-backward): 5 a link.
-// That is 147 instructions at n = 7 and 510 at n = 32. Exchanges are shuffles and
-// shared memory, free beside the FP64 unit. Two instances per warp, one warp per block
+// That is 147 FP64 instructions at n = 7 and 510 at n = 32, counted in the source.
+// Exchanges are shuffles and shared memory; profiled at n = 7, B = 1024 they are what
+// the warps wait for (short scoreboard 3.4 per issue), the FP64 unit 41% busy. Two instances per warp, one warp per block
 // so that blocks spread over the SMs. us, scans / this at B = 1024: n = 7: 29.5 / 10.2,
 // n = 16: 36.4 / 17.2, n = 32: 49.6 / 32.6; at B = 4096: 55 / 22, 134 / 38, 181 / 74. From
 // about 44 instances per SM the one-thread kernel does the work in fewer
