@@ -17,9 +17,11 @@
 // by Horner's rule in 64-bit fractions; the terms below 2^-25 (2^-28) of the leading
 // one in 32 bits, where their rounding costs under 2^-60. First omitted terms:
 // 2^-62 and 2^-61. Then sin r = r - r h in one multiply-add and cos r = 1 - y rounded
-// from its fraction: both within 0.51 ulp of r's sine and cosine, which r's own
-// rounding (one part in 2^53) brings to about 0.8 (the library: 1 to 2).
-// Angles of 2^30 rad or more, infinities and NaN take the library.
+// from its fraction: both within 0.51 ulp of r's sine and cosine. r's own rounding
+// is half an ulp of r, a whole one of a sine that lies in the binade below: at most 1.51
+// ulp in all (the library: up to 2). Seen against 113- and 140-bit values: up to 1.35
+// over one turn, 1.49 up to 2^30 rad, 0.3 on average.
+// The sine of -0 is +0. Angles of 2^30 rad or more, infinities and NaN take the library.
 #pragma once
 #include <cuda_runtime.h>
 
