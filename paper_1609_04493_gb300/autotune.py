@@ -9,15 +9,18 @@ frames with the constants as a kernel parameter and K stored links, or with
 the state of the first links in tensor memory; or the lane-parallel scan with L
 lanes; fleet_batch: persistent CTA shape or one launch per group), and this
 module times the candidates on the caller's own data with CUDA events, keeps
-the fastest, and caches the answer in a JSON file keyed by GPU name, SM count
-and the workload's shape (RDYN_TUNE_CACHE, default ~/.cache/rdyn/tune.json).
+the fastest, and caches the answer in a JSON file keyed by the library's build, GPU
+name, SM count and the workload's shape (RDYN_TUNE_CACHE, default
+~/.cache/rdyn/tune.json): another build's kernels have another winner.
 It only times library calls; it computes nothing itself.
 """
 from __future__ import annotations
 
+import functools
 import json
 import os
 import threading
+import zlib
 
 from . import binding as b
 
@@ -47,6 +50,19 @@ def _store(key, value):
         with open(tmp, "w") as fh:
             json.dump(c, fh, indent=1, sort_keys=True)
         os.replace(tmp, path)
+
+
+@functools.lru_cache(maxsize=4)
+def _crc(path, mtime_ns, size):
+    with open(path, "rb") as fh:
+        return f"{zlib.crc32(fh.read()):08x}"
+
+
+def _build_key():
+    """The loaded library's build: the checksum of its file."""
+    path = b.library_path()
+    st = os.stat(path)
+    return _crc(path, st.st_mtime_ns, st.st_size)
 
 
 def _gpu_key(torch, dev):
@@ -104,7 +120,7 @@ def tune_rnea(model, q, qd, qdd, out=None, reps=5, use_cache=True):
     (variant, {variant: ms})."""
     import torch
 
-    key = f"rnea|{_gpu_key(torch, q.device)}|n={model.n}|B={q.shape[0]}|{q.dtype}"
+    key = f"rnea|{_build_key()}|{_gpu_key(torch, q.device)}|n={model.n}|B={q.shape[0]}|{q.dtype}"
     if use_cache:
         hit = _load_cache().get(key)
         if hit is not None:
@@ -149,15 +165,13 @@ def tune_fleet(plan, q, qd, in2, out=None, reps=3, use_cache=True, flags=0):
     """Fastest (schedule, tune word) for this plan's request mix, every candidate
     run with ``flags`` (e.g. RD_FLEET_FP64_UPDATE) OR-ed into its schedule;
     returns ((schedule, tune), {(schedule, tune): ms}) without the flags."""
-    import zlib
-
     import numpy as np
     import torch
 
     hist = np.bincount(plan.lengths * 2 + plan.kinds, minlength=2 * 130)
     sig = (f"R={plan.R}|J={plan.total_joints}|h={zlib.crc32(hist.tobytes()):08x}|{plan.dtype}"
            f"|f={int(flags):x}")
-    key = f"fleet|{_gpu_key(torch, q.device)}|{sig}"
+    key = f"fleet|{_build_key()}|{_gpu_key(torch, q.device)}|{sig}"
     if use_cache:
         hit = _load_cache().get(key)
         if hit is not None:

@@ -65,3 +65,29 @@ def test_rnea_candidates_cover_the_common_normal_kernels():
         tm = [v for v in cands if (v & 0xfff) == b.RD_VARIANT_SERIAL_DH_TMEM]
         assert bool(tm) == (n <= 32 and n % 4 == 0 and dt != "float64"), (n, dt)
         assert b.RD_VARIANT_AUTO in cands
+
+
+def test_a_pick_lasts_as_long_as_the_library_build(tmp_path, monkeypatch):
+    """A cached winner is taken back for the build it was measured with, and measured
+    anew for another one, whose kernels may rank otherwise."""
+    import types
+
+    import numpy as np
+    import torch
+
+    monkeypatch.setenv("RDYN_TUNE_CACHE", str(tmp_path / "tune.json"))
+    so = tmp_path / "librdyn.so"
+    monkeypatch.setattr(b, "library_path", lambda: str(so))
+    monkeypatch.setattr(autotune, "_gpu_key", lambda torch, dev: "gpu")
+    timed = []
+    monkeypatch.setattr(autotune, "_time", lambda torch, fn, reps: timed.append(1) or float(len(timed)))
+    x = torch.zeros(4, 6)
+    model = types.SimpleNamespace(n=6)
+    plan = types.SimpleNamespace(R=4, total_joints=24, dtype="float32", lengths=np.full(4, 6),
+                                 kinds=np.ones(4, dtype=np.int64))
+    for tune in (lambda: autotune.tune_rnea(model, x, x, x), lambda: autotune.tune_fleet(plan, x, x, x)):
+        for build, fresh in ((b"one", True), (b"one", False), (b"another", True), (b"one", False)):
+            so.write_bytes(build)
+            timed.clear()
+            tune()
+            assert bool(timed) == fresh, build
