@@ -233,18 +233,6 @@ bool aba_use_tri(int n, int B, int flags, bool ext)
     return !ext && B <= 2048;
 }
 
-inline int aba_sms(int device)
-{
-    static std::atomic<int> cache[64];
-    std::atomic<int> &slot = cache[device & 63];
-    int v = slot.load();
-    if (!v) {
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-        slot.store(v);
-    }
-    return v;
-}
-
 // FP64 data: the FP64 unit does about 150 instructions a link for ten instances
 // instead of 415 for 32, so three lanes lead while two blocks of thirty per SM hold
 // the batch and one warp per instance (n >= 48, B <= 512) does not. us, one thread / three
@@ -257,7 +245,7 @@ inline bool aba_use_trio_f64(const rd_model *m, int B, int flags)
     if (flags & (RD_ABA_THREAD_PER_INSTANCE | RD_ABA_WARP_PER_INSTANCE | RD_ABA_TWO_WARPS |
                  RD_ABA_THREE_WARPS | RD_ABA_JOINT_FRAMES))
         return false;
-    return m->n >= 3 && !aba_use_warp<double>(m->n, B, flags) && (long long)B <= 60LL * aba_sms(m->device);
+    return m->n >= 3 && !aba_use_warp<double>(m->n, B, flags) && (long long)B <= 60LL * rd_sm_count(m->device);
 }
 
 // Three lanes per instance (aba_trio.cuh): by flag, else for FP32 data with
@@ -276,7 +264,7 @@ inline bool aba_use_trio(const rd_model *m, int B, int flags, bool ext)
     if (flags & (RD_ABA_THREAD_PER_INSTANCE | RD_ABA_WARP_PER_INSTANCE | RD_ABA_JOINT_FRAMES |
                  RD_ABA_SCANS_IN_DTYPE | RD_ABA_FP64_UPDATE | RD_ABA_TEST_WITHHOLD))
         return false;
-    return m->n >= 3 && (long long)B <= (ext ? 160LL : 120LL) * aba_sms(m->device);
+    return m->n >= 3 && (long long)B <= (ext ? 160LL : 120LL) * rd_sm_count(m->device);
 }
 
 template <typename T>

@@ -54,6 +54,8 @@ inline void rd_note_rnea(int kernel, int block, int stored, int register_links =
     g_rd_last_rnea.register_links = register_links;
     g_rd_last_rnea.ring_chunks = ring_chunks;
 }
+// SMs of a device, asked once (152, a GB300's, if the device does not say)
+int rd_sm_count(int device);
 int rd_fail(int code, const char *fmt, ...);
 int rd_cuda_fail(cudaError_t e, const char *what);
 void rd_convert_base(const rd_model *m, const double *base, double out[18]);

@@ -14,6 +14,7 @@
 // All of this runs once, in double precision, on the host.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -148,6 +149,21 @@ bool psd3(const double I[3][3])
 }
 
 }  // namespace
+
+int rd_sm_count(int device)
+{
+    static std::atomic<int> cache[64];
+    std::atomic<int> &slot = cache[device & 63];
+    int v = slot.load();
+    if (v == 0) {
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || v <= 0) {
+            cudaGetLastError();  // the next launch's check is not to find it
+            return 152;
+        }
+        slot.store(v);
+    }
+    return v;
+}
 
 extern "C" int rd_version(void) { return 100; }
 

@@ -152,14 +152,6 @@ int dh_device_attr(int device, cudaDeviceAttr attr, int fallback)
     return v;
 }
 
-int dh_sms(int device)
-{
-    static std::atomic<int> cache[64];
-    const int d = device & 63;
-    if (cache[d].load() == 0) cache[d].store(dh_device_attr(device, cudaDevAttrMultiProcessorCount, 1));
-    return cache[d].load();
-}
-
 // Default K for the parameter-constant kernel (32-thread blocks). On GB300 at
 // B = 65536 the fastest K at every length was the largest that still leaves 7
 // blocks per SM, so the batch runs in at most two waves (n = 16: K = 16, 10.8 us;
@@ -169,12 +161,11 @@ int dh_sms(int device)
 template <typename T>
 int dhp_default_k(const rd_model *m, int B)
 {
-    static std::atomic<int> smem_sm[64], sms[64];
+    static std::atomic<int> smem_sm[64];
     const int d = m->device & 63;
-    if (smem_sm[d].load() == 0) {
+    if (smem_sm[d].load() == 0)
         smem_sm[d].store(dh_device_attr(m->device, cudaDevAttrMaxSharedMemoryPerMultiprocessor, 100 * 1024));
-        sms[d].store(dh_device_attr(m->device, cudaDevAttrMultiProcessorCount, 1));
-    }
+    const long long sms = rd_sm_count(m->device);
     const int n = m->n;
     auto blocks_per_sm = [&](int K) {
         const size_t per_block = dhp_smem_per_thread<T>(n, K) * 32 + 1024;  // + the block's reserve
@@ -185,7 +176,7 @@ int dhp_default_k(const rd_model *m, int B)
     int best = 0;
     for (int K = 0; K <= n; K += 4) {
         const int per_sm = blocks_per_sm(K);
-        if (per_sm >= 7 || (long long)per_sm * sms[d].load() >= blocks) best = K;
+        if (per_sm >= 7 || (long long)per_sm * sms >= blocks) best = K;
     }
     return best;
 }
@@ -236,7 +227,7 @@ void dhp_default_kr(const rd_model *m, int B, int &K, int &RL, int &stages)
             &per_sm, rnea_dhp_kernel<float, 32, 32, TRIG, 4, 2>, 32, smem);
         slot.store(per_sm + 1);
     }
-    const long long sms = dh_sms(m->device);
+    const long long sms = rd_sm_count(m->device);
     if ((long long)per_sm * sms >= 2 * ((long long)(B + 31) / 32)) {
         RL = 4;
         stages = 2;
@@ -275,7 +266,7 @@ int launch_dhp_ragged(const rd_model *m, int B, const void *q, const void *qd, c
                 dhp_smem_per_thread<float>(n, n, 4, 2) * 32);
             slot.store(per_sm + 1);
         }
-        const long long sms = dh_sms(m->device);
+        const long long sms = rd_sm_count(m->device);
         if (2 * (long long)per_sm * sms < (long long)(B + 31) / 32) RL = 8;
     }
     const size_t smem = dhp_smem_per_thread<float>(n, n, RL, 2) * 32;
@@ -409,10 +400,7 @@ int launch_dht_k(const rd_model *m, int K, int TL, int B, const void *q, const v
     for (int k = m->n * kDhConsts; k < 32 * kDhConsts; ++k) pc.c[k] = 0.0f;
     // four blocks per SM, each with an equal share of the batch in rounds of
     // at most 128 instances
-    static std::atomic<int> sms[64];
-    const int d = m->device & 63;
-    if (sms[d].load() == 0) sms[d].store(dh_device_attr(m->device, cudaDevAttrMultiProcessorCount, 1));
-    const long long max_grid = 4LL * sms[d].load(), min_grid = ((long long)B + 31) / 32;
+    const long long max_grid = 4LL * rd_sm_count(m->device), min_grid = ((long long)B + 31) / 32;
     const long long grid = max_grid < min_grid ? max_grid : min_grid;
     const long long per_block = ((long long)B + grid - 1) / grid;
     const long long rounds = (per_block + kDhtThreads - 1) / kDhtThreads;

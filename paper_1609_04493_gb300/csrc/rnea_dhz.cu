@@ -41,10 +41,8 @@ int launch_dhz_k(const rd_model *m, int B, const float *q, const float *qd, cons
     // 160, 6: 164, 8: 158, 13 (all slabs resident at once): 179; the staged
     // copies take 209
     constexpr int per_sm = 8;
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
-    const long long slabs = (B + BLOCK - 1) / BLOCK;
-    const unsigned grid = (unsigned)(slabs < (long long)sms * per_sm ? slabs : (long long)sms * per_sm);
+    const long long slabs = (B + BLOCK - 1) / BLOCK, most = (long long)per_sm * rd_sm_count(m->device);
+    const unsigned grid = (unsigned)(slabs < most ? slabs : most);
     rd_note_rnea(RD_RNEA_KERNEL_DH_HOST, BLOCK, 0);
     kern<<<grid, BLOCK, smem, stream>>>(pc, n, B, q, qd, qdd, tau, bp);
     cudaError_t e = cudaGetLastError();

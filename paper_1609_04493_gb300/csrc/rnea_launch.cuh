@@ -42,18 +42,6 @@ int max_smem_optin(int device)
     return v;
 }
 
-int sm_count(int device)
-{
-    static std::atomic<int> cache[64];
-    const int d = device & 63;
-    int v = cache[d].load();
-    if (v == 0) {
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) v = 1;
-        cache[d].store(v);
-    }
-    return v;
-}
-
 // Raise a kernel's dynamic shared-memory limit once per device.
 template <typename K>
 cudaError_t allow_smem(K kern, int device, std::atomic<uint64_t> &done)
@@ -310,6 +298,7 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     const int regstate = 4 * ((variant >> 28) & 0x7);   // RD_TUNE_REG_STATE_LINKS
     const int stages = (variant & RD_TUNE_TWO_STAGE_RING) ? 2 : kStages;
     variant &= 0xfff;
+    const long long sms = rd_sm_count(m->device);
     const bool dhp_rows = sizeof(T) == 4 && n % 4 == 0 && n <= 128 && aligned16(q) &&
                           aligned16(qd) && aligned16(qdd) && aligned16(tau);
     // rows of any length and alignment, untuned, for the common-normal kernel
@@ -327,8 +316,7 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
         // lanes at 6000 (634 / 959).
         const bool fits = rd_rnea_dhp_f64_fits(m);
         const long long per_sm = n == 1 ? 12 : n <= 3 ? 22 : 44;
-        if (variant == RD_VARIANT_AUTO && untuned && (fits || B > 152 * 32) &&
-            B <= per_sm * sm_count(m->device))
+        if (variant == RD_VARIANT_AUTO && untuned && (fits || B > 32 * sms) && B <= per_sm * sms)
             return rd_rnea_wide_f64(m, B, q, qd, qdd, tau, base18, s);
         if (variant == RD_VARIANT_AUTO && untuned && fits)
             return rd_rnea_dh_f64(m, B, q, qd, qdd, tau, base18, 1, 0, 0, RD_DHP_AUTO_F64, 0, 0,
@@ -336,7 +324,7 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     }
     // the common-normal kernel of the next branch overtakes the scans sooner
     // (n = 32: 7.5 us against 9.3 at B = 4096; 6.9 against 5.0 at B = 1024)
-    if (variant == RD_VARIANT_AUTO && B <= (dhp_rows || ragged ? 2048 : 152 * 32) && n <= 128) {
+    if (variant == RD_VARIANT_AUTO && B <= (dhp_rows || ragged ? 2048 : 32 * sms) && n <= 128) {
         // Fewer instances than one warp per SM: the serial recursion leaves the
         // GPU idle, and splitting each chain over lanes (the scans of Sec. III)
         // cuts latency. Measured: n = 32, B = 1024 FP32 5.1 us with 16 lanes vs 8.4

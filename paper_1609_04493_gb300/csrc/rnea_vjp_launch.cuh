@@ -230,7 +230,7 @@ int launch_vjp_dh(const rd_model *m, int B, const void *q, const void *qd, const
         }
     }
     // small batches: 32-thread blocks spread the few warps over more SMs
-    const bool small = B <= 152 * 128;
+    const bool small = B <= 128LL * rd_sm_count(m->device);
     if (m->n <= 32)
         return small ? launch_vjp_dh_k<T, 32, 32, MODE, TRIG>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s)
                      : launch_vjp_dh_k<T, 32, 64, MODE, TRIG>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
@@ -281,7 +281,7 @@ int launch_vjp_any(const rd_model *m, int B, const void *q, const void *qd, cons
     // 8192 and 65536: n = 7: 7.7 / 8.9, 13.3 / 16.1; 14: 12.4 / 12.0, 26.0 / 28.3; 19: 17.6
     // / 14.2, 36.2 / 37.3; 21: 19.1 / 14.7, 40.8 / 39.8; 25: 21.8 / 16.3, 49.0 / 43.2; 63 at
     // 65536: 139 / 104).
-    const bool pays = sizeof(T) == 8 || m->n >= 21 || (m->n >= 14 && B <= 152 * 128);
+    const bool pays = sizeof(T) == 8 || m->n >= 21 || (m->n >= 14 && B <= 128LL * rd_sm_count(m->device));
     if (!joint_frames && pays && m->n <= 128 && split <= 0) {
         if (sizeof(T) == 4 && fast)
             return launch_vjp_ragged<T, MODE, kTrigSfu>(m, B, q, qd, qdd, w, gq, gqd, gqdd, ws, base18, s);
