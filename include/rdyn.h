@@ -443,7 +443,8 @@ enum rd_schedule {
  * (0 = library default: 4 CTAs per SM of 128 threads, or of 64 where an RD_F32 plan
  * has few requests). Forward-dynamics requests of RD_F32 plans with double-float
  * updates run three lanes per request (as RD_ABA_THREE_LANES), ten per pair of
- * warps. */
+ * warps, or one thread per request where a plan has so many of like length that this is
+ * faster; the plan decides, so every schedule and shape gives the same bits. */
 #define RD_FLEET_TUNE(log2_threads, ctas_per_sm) (((log2_threads) << 8) | (ctas_per_sm))
 /* OR-ed into the tune word of the persistent schedule: groups of 32 sorted
  * requests that start with a forward-dynamics chain of at least min_links links

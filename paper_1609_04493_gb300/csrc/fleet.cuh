@@ -244,10 +244,10 @@ __device__ __forceinline__ void fleet_request_pair(const FleetArgs<T, D> &a, int
 }
 
 // ---- forward dynamics with three lanes per request (aba_trio.cuh), FP32 data
-// with double-float updates: units of ten sorted positions, two warps each (the
+// with double-float updates, in the plans that fleet_rule.h picks: units of ten sorted positions, two warps each (the
 // bias sweeps; the inertias and the solves), or one warp doing both in turn. A
 // unit's bias sweeps run in double-float if any of its requests' groups of 32
-// asks for it, so a request's arithmetic depends on its position alone, not on
+// asks for it, so a request's arithmetic depends on the plan alone, not on
 // the schedule. 20 000 requests of 6..100 links (4000 forward dynamics): 944 us with
 // one thread per request, 335 now; 1000 requests: 790 / 257; 100 000: 1150 / 594.
 // Bound by the longest chains' dependent updates (100 links: 224 us alone).

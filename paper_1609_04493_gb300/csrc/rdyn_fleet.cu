@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "fleet.cuh"
+#include "fleet_rule.h"
 #include "rdyn_internal.h"
 
 struct rd_fleet {
@@ -47,8 +48,10 @@ struct rd_plan {
     // starts it (0 when it starts with inverse dynamics), for the two-warp
     // schedule's threshold
     std::vector<int> group_fd_n;
-    // three-lane forward dynamics (FP32 plans): the number of forward-dynamics
+    // three-lane forward dynamics (FP32 plans, where fleet_rule.h takes it; in every
+    // schedule, so that they agree bit for bit): the number of forward-dynamics
     // requests, and the workspace per ten sorted positions
+    bool lanes = false;
     int fd_count = 0;
     long long *unit_ws = nullptr, *unit_wz = nullptr;
     unsigned char *ws = nullptr;
@@ -234,11 +237,15 @@ extern "C" int rd_plan_create(const rd_fleet *f, int R, const int *robot, const 
     // (the positions are sorted, so it is the unit's longest chain)
     int fd_count = 0;
     while (fd_count < R && kind[order[fd_count]] == RD_REQ_FD) ++fd_count;
+    std::vector<int> fd_n, id_n;
+    for (int k = 0; k < R; ++k) (k < fd_count ? fd_n : id_n).push_back(f->n[robot[order[k]]]);
+    const bool lanes = dtype == RD_F32 && rd_fleet_takes_lanes(fd_n, id_n, ext_groups, rdyn::kTrioPerWarp,
+                                                               rd_sm_count(f->device));
     std::vector<long long> uws, uwz;
-    if (dtype == RD_F32) {
+    if (lanes) {
         size_t at = 0;
         for (int k = 0; k < fd_count; k += rdyn::kTrioPerWarp) {
-            const size_t nmax = (size_t)f->n[robot[order[k]]];
+            const size_t nmax = (size_t)fd_n[k];
             uws.push_back((long long)at);
             at += (nmax * ((k >> 5) < ext_groups ? 16 : 10) * rdyn::kTrioPerWarp * 4 + 255) & ~(size_t)255;
             uwz.push_back((long long)at);
@@ -248,6 +255,7 @@ extern "C" int rd_plan_create(const rd_fleet *f, int R, const int *robot, const 
     }
     rd_plan *p = new (std::nothrow) rd_plan();
     if (!p) return rd_fail(RD_ERR_ALLOC, "rd_plan_create: host allocation failed");
+    p->lanes = lanes;
     p->fd_count = fd_count;
     p->fleet = f;
     p->dtype = dtype;
@@ -383,8 +391,14 @@ int run_fleet(const rd_plan *p, const void *q, const void *qd, const void *in2, 
             return rd_fail(RD_ERR_ARG, "fleet_batch: %d threads per block", threads);
         e = cudaMemsetAsync(p->counter, 0, 2 * sizeof(int), s);
         if (e != cudaSuccess) return rd_cuda_fail(e, "fleet_batch: counter reset");
-        if constexpr (std::is_same<D, rdyn::DF>::value) {
-            // By default one pair of warps per block where every unit then has
+        bool lanes = false;
+        if constexpr (std::is_same<D, rdyn::DF>::value) lanes = p->lanes;
+        if (!lanes) {
+            // 512 threads of 234 registers do not fit an SM: two blocks of 256
+            const int halves = std::is_same<D, rdyn::DF>::value && threads == 512 ? 2 : 1;
+            rdyn::fleet_persistent_kernel<T, D><<<p->sms * per_sm * halves, threads / halves, 0, s>>>(a);
+        } else if constexpr (std::is_same<D, rdyn::DF>::value) {
+            // Three lanes per request. By default one pair of warps per block where every unit then has
             // a pair at once and the inverse-dynamics requests are few: the other
             // two warps would only take issue slots from the longest chains, which
             // set the time (us, 128 threads / 64: 20 000 requests of 6..100 links 377 /
@@ -405,8 +419,6 @@ int run_fleet(const rd_plan *p, const void *q, const void *qd, const void *in2, 
                 configured.fetch_or(bit);
             }
             rdyn::fleet_trio_kernel<<<p->sms * per_sm, threads, smem, s>>>(a);
-        } else {
-            rdyn::fleet_persistent_kernel<T, D><<<p->sms * per_sm, threads, 0, s>>>(a);
         }
     } else if (schedule == RD_SCHED_PER_GROUP) {
         // one launch per group, spread over side streams that fork from and
@@ -419,9 +431,12 @@ int run_fleet(const rd_plan *p, const void *q, const void *qd, const void *in2, 
         for (const auto &g : p->groups) {
             const int len = g.second - g.first;
             if constexpr (std::is_same<D, rdyn::DF>::value) {
-                if (g.first < p->fd_count) {
+                if (p->lanes && g.first < p->fd_count) {
                     const int units = (g.second - 1) / rdyn::kTrioPerWarp - g.first / rdyn::kTrioPerWarp + 1;
                     rdyn::fleet_trio_range_kernel<<<units, 64, 0, p->side[k]>>>(a, g.first, g.second);
+                } else if (g.first < p->fd_count) {
+                    rdyn::fleet_range_kernel<T, D><<<(len + 127) / 128, 128, 0, p->side[k]>>>(
+                        a, g.first, g.second);
                 } else {
                     rdyn::fleet_id_range_kernel<T, D><<<(len + 127) / 128, 128, 0, p->side[k]>>>(
                         a, g.first, g.second);
