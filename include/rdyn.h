@@ -110,9 +110,13 @@ enum rd_status {
  * instance (one per axis; ten instances per warp), beside a warp for the bias
  * sweeps. Same exclusions. The library's choice for n >= 3 while the batch is
  * resident at once (RD_F64: B <= 60 per SM where one warp per instance does not lead;
- * RD_F32: 120, or 160 with double-float bias sweeps), where for RD_F32 it also serves RD_ABA_TWO_WARPS and RD_ABA_THREE_WARPS (the same split of the work,
- * results to rounding). */
+ * RD_F32: 120, or 160 with double-float bias sweeps). Where it took the place of two
+ * or of three warps in that choice, it also serves an RD_F32 call that names that
+ * one of the two (results to rounding) unless RD_ABA_EXACT_MAPPING is set. */
 #define RD_ABA_THREE_LANES 0x200
+/* aba_batch flag, with a mapping flag: run that mapping itself at every n and B (see
+ * RD_ABA_THREE_LANES; the other mapping flags are always taken as they are). */
+#define RD_ABA_EXACT_MAPPING 0x400
 /* aba_batch test hook, only with RD_ABA_TWO_WARPS: the articulated-inertia warp
  * withholds its per-link announcements, so every wait of the other warp runs
  * out (one bounded wait per instance, a quarter of a second or more) and every

@@ -249,21 +249,30 @@ inline bool aba_use_trio_f64(const rd_model *m, int B, int flags)
 }
 
 // Three lanes per instance (aba_trio.cuh): by flag, else for FP32 data with
-// double-float updates (also where the two- or three-warp form is asked for, which
-// it supersedes there) while the batch is resident at once, which is what the
+// double-float updates while the batch is resident at once, which is what the
 // split is for: four blocks per SM (thirty instances each, or twenty with the
 // double-float bias sweeps, where two such waves still win). Times in us on
 // GB300, the mapping taken otherwise / three lanes: n = 7: 17.6 / 13.2 at B = 1024, 34.9 / 23.7 at
 // 18240, 35.7 / 38.1 at 24000; n = 64: 346 / 217 at 18240, 360 / 355 at 24000, 352 /
 // 440 at 32768; n = 100: 822 / 704 at 16384, 990 / 852 at 24000, 938 / 1197 at
 // 32768. Below three links nothing is left to split (n = 2: 5.2 / 5.3 at B = 64,
-// 7.5 / 8.0 at 16384).
+// 7.5 / 8.0 at 16384). A flag for two or for three warps is served too where that one is
+// the mapping this rule replaces, as the choice without a flag and the flag for it
+// agree bit for bit; RD_ABA_EXACT_MAPPING takes the named kernel there as well.
 inline bool aba_use_trio(const rd_model *m, int B, int flags, bool ext)
 {
     if (flags & RD_ABA_THREE_LANES) return true;
     if (flags & (RD_ABA_THREAD_PER_INSTANCE | RD_ABA_WARP_PER_INSTANCE | RD_ABA_JOINT_FRAMES |
                  RD_ABA_SCANS_IN_DTYPE | RD_ABA_FP64_UPDATE | RD_ABA_TEST_WITHHOLD))
         return false;
+    const int warps = flags & (RD_ABA_TWO_WARPS | RD_ABA_THREE_WARPS);
+    if (warps) {
+        const int rest = flags & ~warps;
+        const int replaced = aba_use_tri<float>(m->n, B, rest, ext)   ? RD_ABA_THREE_WARPS
+                             : aba_use_pair<float>(m->n, B, rest)     ? RD_ABA_TWO_WARPS
+                                                                      : 0;
+        if ((flags & RD_ABA_EXACT_MAPPING) || warps != replaced) return false;
+    }
     return m->n >= 3 && (long long)B <= (ext ? 160LL : 120LL) * rd_sm_count(m->device);
 }
 
@@ -291,6 +300,8 @@ int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const 
                                        "RD_ABA_THREE_WARPS, RD_ABA_THREE_LANES and "
                                        "RD_ABA_THREAD_PER_INSTANCE exclude one another, and the "
                                        "first four RD_ABA_JOINT_FRAMES and RD_ABA_SCANS_IN_DTYPE");
+        if ((flags & RD_ABA_EXACT_MAPPING) && !maps)
+            return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_EXACT_MAPPING needs a mapping flag");
         if ((flags & RD_ABA_THREE_LANES) && sizeof(T) == 4 && (flags & RD_ABA_FP64_UPDATE))
             return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_THREE_LANES takes RD_F64 data, or RD_F32 data with "
                                        "double-float updates");
