@@ -285,6 +285,20 @@ int launch_regstate(const rd_model *m, int block, int reglinks, int B, const voi
                                "%d register links", block, reglinks);
 }
 
+// FP32 rows of any length and alignment: the largest batch for which the lane-parallel
+// scans lead over the common-normal kernel. Their time steps up with every eight
+// instances an SM and every sixteen links, at which it is fullest. us, scans / common-normal
+// at B = 2432 (sixteen an SM): n = 9: 4.3 / 4.2, 13: 4.5 / 4.7, 15: 4.5 / 5.3, 17: 5.6 / 5.5, 25: 6.1 /
+// 6.8, 31: 6.5 / 8.0, 33: 9.0 / 8.2, 45: 10.6 / 10.3, 63: 13.2 / 13.7, 65: 14.2 / 13.8, 79: 16.1 / 16.9,
+// 99: 19.1 / 20.9, 127: 23.2 / 26.3; at 2433: 25: 7.0 / 6.9, 99: 24.8 / 20.8; at 3648: 15: 5.3 /
+// 5.6, 31: 8.0 / 8.3, at 3649: 5.9 / 5.6, 8.7 / 8.3.
+inline long long ragged_scan_most(int n, long long sms)
+{
+    if (n == 15 || n == 31) return 24 * sms;
+    if ((n >= 10 && n <= 32) || n == 62 || n == 63 || n > 65) return 16 * sms;
+    return 2048;
+}
+
 template <typename T>
 int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void *qdd, void *tau,
              const double *base18, int variant, cudaStream_t s)
@@ -301,9 +315,11 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     const long long sms = rd_sm_count(m->device);
     const bool dhp_rows = sizeof(T) == 4 && n % 4 == 0 && n <= 128 && aligned16(q) &&
                           aligned16(qd) && aligned16(qdd) && aligned16(tau);
-    // rows of any length and alignment, untuned, for the common-normal kernel
+    // rows of any length and alignment, untuned, for the common-normal kernel. One or two
+    // links leave it no chunk to stream (us, joint frames / it: n = 1, B = 65536: 2.6 / 3.1;
+    // n = 2: 3.2 / 3.6; n = 3: 4.0 / 4.0)
     const bool untuned = (!block || block == 32) && !reglinks && !regstate && stages == kStages;
-    const bool ragged = sizeof(T) == 4 && !dhp_rows && n <= 128 && untuned;
+    const bool ragged = sizeof(T) == 4 && !dhp_rows && n >= 3 && n <= 128 && untuned;
     if constexpr (sizeof(T) == 8) {
         // FP64, untuned: sixteen lanes per instance (rnea_wide.cuh) while that takes
         // fewer cycles of the FP64 unit than one thread per instance, whose time
@@ -324,7 +340,8 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     }
     // the common-normal kernel of the next branch overtakes the scans sooner
     // (n = 32: 7.5 us against 9.3 at B = 4096; 6.9 against 5.0 at B = 1024)
-    if (variant == RD_VARIANT_AUTO && B <= (dhp_rows || ragged ? 2048 : 32 * sms) && n <= 128) {
+    const long long scan_most = dhp_rows ? 2048 : ragged ? ragged_scan_most(n, sms) : 32 * sms;
+    if (variant == RD_VARIANT_AUTO && B <= scan_most && n <= 128) {
         // Fewer instances than one warp per SM: the serial recursion leaves the
         // GPU idle, and splitting each chain over lanes (the scans of Sec. III)
         // cuts latency. Measured: n = 32, B = 1024 FP32 5.1 us with 16 lanes vs 8.4
