@@ -569,6 +569,11 @@ int rd_rnea_last_config(int *kernel, int *block, int *stored_links);
  * after any other kernel. Errors: RD_ERR_ARG (null output). */
 int rd_rnea_last_state_layout(int *register_links, int *ring_chunks);
 
+/* The mapping of the calling thread's last aba_batch launch (a diagnostic): its mapping
+ * flag (RD_ABA_THREAD_PER_INSTANCE, ..._WARP_PER_INSTANCE, ..._TWO_WARPS,
+ * ..._THREE_WARPS, ..._THREE_LANES), or RD_ABA_JOINT_FRAMES; 0 before the first. */
+int rd_aba_last_mapping(void);
+
 /* Message for the last error on the calling thread ("" if none). */
 const char *rd_last_error(void);
 

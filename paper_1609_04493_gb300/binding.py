@@ -138,6 +138,8 @@ def load(build_if_missing=True):
         IP = ctypes.POINTER(ctypes.c_int)
         lib.rd_rnea_last_config.argtypes = [IP, IP, IP]
         lib.rd_rnea_last_config.restype = I
+        lib.rd_aba_last_mapping.argtypes = []
+        lib.rd_aba_last_mapping.restype = I
         lib.rd_rnea_last_state_layout.argtypes = [IP, IP]
         lib.rd_rnea_last_state_layout.restype = I
         _lib = lib
@@ -175,6 +177,11 @@ def rnea_last_config():
     k, b, s = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     _check(lib.rd_rnea_last_config(ctypes.byref(k), ctypes.byref(b), ctypes.byref(s)))
     return k.value, b.value, s.value
+
+
+def aba_last_mapping():
+    """The mapping flag of this thread's last aba_batch launch (rd_aba_last_mapping)."""
+    return load().rd_aba_last_mapping()
 
 
 def rnea_last_state_layout():

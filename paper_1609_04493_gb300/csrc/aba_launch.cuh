@@ -310,13 +310,18 @@ int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const 
     if (withhold && !(flags & RD_ABA_TWO_WARPS))
         return rd_fail(RD_ERR_ARG, "aba_batch: RD_ABA_TEST_WITHHOLD needs RD_ABA_TWO_WARPS");
     if constexpr (sizeof(T) == 4) {
-        if (aba_use_trio(m, B, flags, ext))
+        if (aba_use_trio(m, B, flags, ext)) {
+            g_rd_last_aba = RD_ABA_THREE_LANES;
             return rd_aba_trio_f32(m, B, q, qd, tau, qdd, status, ws, base18, ext, s);
+        }
     } else {
-        if (aba_use_trio_f64(m, B, flags))
+        if (aba_use_trio_f64(m, B, flags)) {
+            g_rd_last_aba = RD_ABA_THREE_LANES;
             return rd_aba_trio_f64(m, B, q, qd, tau, qdd, status, ws, base18, s);
+        }
     }
     if (aba_use_tri<T>(m->n, B, flags, ext)) {
+        g_rd_last_aba = RD_ABA_THREE_WARPS;
         if constexpr (sizeof(T) == 4)
             return rd_aba_tri_f32(m, B, q, qd, tau, qdd, status, ws, base18,
                                   (flags & RD_ABA_FP64_UPDATE) != 0, ext, s);
@@ -324,6 +329,7 @@ int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const 
             return rd_aba_tri_f64(m, B, q, qd, tau, qdd, status, ws, base18, s);
     }
     if (aba_use_pair<T>(m->n, B, flags)) {
+        g_rd_last_aba = RD_ABA_TWO_WARPS;
         if constexpr (sizeof(T) == 4)
             return rd_aba_pair_f32(m, B, q, qd, tau, qdd, status, ws, base18,
                                    (flags & RD_ABA_FP64_UPDATE) != 0, ext, withhold, s);
@@ -331,12 +337,14 @@ int aba_dispatch(const rd_model *m, int B, const void *q, const void *qd, const 
             return rd_aba_pair_f64(m, B, q, qd, tau, qdd, status, ws, base18, withhold, s);
     }
     if (aba_use_warp<T>(m->n, B, flags)) {
+        g_rd_last_aba = RD_ABA_WARP_PER_INSTANCE;
         if constexpr (sizeof(T) == 4)
             return rd_aba_warp_f32(m, B, q, qd, tau, qdd, status, base18,
                                    (flags & RD_ABA_FP64_UPDATE) != 0, ext, s);
         else
             return rd_aba_warp_f64(m, B, q, qd, tau, qdd, status, base18, s);
     }
+    g_rd_last_aba = flags & RD_ABA_JOINT_FRAMES ? RD_ABA_JOINT_FRAMES : RD_ABA_THREAD_PER_INSTANCE;
     const bool vec = m->n % 4 == 0 && aba_aligned16(q) && aba_aligned16(qd) &&
                      aba_aligned16(tau) && aba_aligned16(qdd);
     if (vec && m->n <= 64 && !ext && !(flags & RD_ABA_JOINT_FRAMES)) {

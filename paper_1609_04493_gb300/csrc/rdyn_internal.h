@@ -45,6 +45,7 @@ struct RdLaunchConfig {
     int kernel = 0, block = 0, stored_links = 0, register_links = 0, ring_chunks = 0;
 };
 extern thread_local RdLaunchConfig g_rd_last_rnea;
+extern thread_local int g_rd_last_aba;  // rd_aba_last_mapping
 inline void rd_note_rnea(int kernel, int block, int stored, int register_links = 0,
                          int ring_chunks = 0)
 {

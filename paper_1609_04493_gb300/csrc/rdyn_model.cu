@@ -27,6 +27,9 @@
 
 thread_local std::string g_rd_error;
 thread_local RdLaunchConfig g_rd_last_rnea;
+thread_local int g_rd_last_aba;
+
+extern "C" int rd_aba_last_mapping(void) { return g_rd_last_aba; }
 
 extern "C" int rd_rnea_last_config(int *kernel, int *block, int *stored_links)
 {
