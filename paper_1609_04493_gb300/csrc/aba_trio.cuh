@@ -353,6 +353,7 @@ __device__ __forceinline__ int aba_trio_solve(const D *__restrict__ sd, int n, i
                                               int b, const TrioLane &L, TrioShared<D> &sh,
                                               TrioRing<D, TB> &rg)
 {
+    static_assert(std::is_same<D, DF>::value || std::is_same<D, T>::value, "FP32 data: double-float");
     using S = decltype(dscalar<D>(TB(0)));
     const int k = L.k, k1 = L.k1, k2 = L.k2;
     D *const own = &sh.x[threadIdx.x & 31];
@@ -386,20 +387,14 @@ __device__ __forceinline__ int aba_trio_solve(const D *__restrict__ sd, int n, i
         D uv, uw, iom, t;  // t: tau_hat, then c_hat
         S c, s;
     };
-    auto take = [&](int u, bool second) -> SolveIn {
+    auto take = [&](int u) -> SolveIn {
         __pipeline_wait_prior(kTrioRing - 2);
         const int slot = u % kTrioRing;
         SolveIn r;
         r.uv = rg.v[slot][0][lane];
         r.uw = rg.v[slot][1][lane];
         r.iom = rg.v[slot][2][lane];
-        if constexpr (std::is_same<D, double>::value && sizeof(T) == 4) {
-            // FP32 data: tau_hat is a pair of floats beside c_hat in D
-            const DF p = *reinterpret_cast<const DF *>(&rg.v[slot][3][lane]);
-            r.t = second ? rg.v[slot][3][lane] : dcvt<D>(p);
-        } else {
-            r.t = rg.v[slot][3][lane];
-        }
+        r.t = rg.v[slot][3][lane];
         r.c = dscalar<D>(rg.cs[slot][0][lane]);
         r.s = dscalar<D>(rg.cs[slot][1][lane]);
         return r;
@@ -417,7 +412,7 @@ __device__ __forceinline__ int aba_trio_solve(const D *__restrict__ sd, int n, i
         const D *r = sd + ii * kAbaDh64;
         const int u = nmax - 1 - i;
         if (RAGGED && ii > 0) prefetch_l1(sd + (ii - 1) * kAbaDh64);
-        const SolveIn cur = take(u, false);
+        const SolveIn cur = take(u);
         fetch(u + kTrioRing - 1, i - (kTrioRing - 1), false);
         const S c = cur.c, s = cur.s;
         const D ca = r[0], sa = r[1];
@@ -460,7 +455,7 @@ __device__ __forceinline__ int aba_trio_solve(const D *__restrict__ sd, int n, i
         const int ii = !RAGGED || in ? i : n - 1;
         const D *r = sd + ii * kAbaDh64;
         if (RAGGED && ii + 1 < n) prefetch_l1(sd + (ii + 1) * kAbaDh64);
-        const SolveIn cur = take(i, true);
+        const SolveIn cur = take(i);
         fetch(i + kTrioRing - 1, i + kTrioRing - 1, true);
         const S c = cur.c, s = cur.s;
         const D ca = r[0], sa = r[1];

@@ -263,15 +263,13 @@ __device__ __forceinline__ To dcvt(From x)
 }
 
 // A plain factor (the sine or cosine of a joint angle) beside values of type D:
-// an FP32 factor stays a float next to double-floats (its products take one
-// multiply-add less), and becomes a double next to doubles.
+// an FP32 factor stays a float next to double-floats: its products take one
+// multiply-add less.
 template <typename D>
 struct DScalar;
 template <>
 struct DScalar<double> {
-    __device__ __forceinline__ static double from(float x) { return (double)x; }
     __device__ __forceinline__ static double from(double x) { return x; }
-    __device__ __forceinline__ static double from(DF x) { return (double)x.hi + (double)x.lo; }
 };
 template <>
 struct DScalar<DF> {
