@@ -108,9 +108,9 @@ enum rd_status {
 /* aba_batch flag, RD_F64 data or RD_F32 data with double-float updates: the
  * articulated-inertia recursion and the solves spread over three lanes per
  * instance (one per axis; ten instances per warp), beside a warp for the bias
- * sweeps. Same exclusions. The library's choice for n >= 3 while the batch is
- * resident at once (RD_F64: B <= 60 per SM where one warp per instance does not lead;
- * RD_F32: 120, or 160 with double-float bias sweeps). Where it took the place of two
+ * sweeps. Same exclusions. The library's choice for n >= 3 and batches of one or two
+ * waves of its blocks (RD_F64: B <= 60 per SM where one warp per instance does not lead;
+ * RD_F32: 120, or 160 with double-float bias sweeps, less for some lengths). Where it took the place of two
  * or of three warps in that choice, it also serves an RD_F32 call that names that
  * one of the two (results to rounding) unless RD_ABA_EXACT_MAPPING is set. */
 #define RD_ABA_THREE_LANES 0x200

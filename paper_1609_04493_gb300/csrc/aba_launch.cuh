@@ -192,6 +192,9 @@ bool aba_use_warp(int n, int B, int flags)
     return B <= (fp64 || n < 96 ? 512 : 1024);
 }
 
+// Largest batch of the two-warp mapping with double-float updates.
+constexpr int kAbaPairMost = 16384;
+
 // Two warps per 32 instances: by flag, else for FP32 data where the measured
 // times favour it over one thread per instance (double-float updates, thread /
 // pair: n = 16: 1.25 at B = 1024, 1.04 at 16384, 0.80 at 65536; n = 64: 1.31 /
@@ -207,7 +210,7 @@ bool aba_use_pair(int n, int B, int flags)
                                     RD_ABA_SCANS_IN_DTYPE)))
         return false;
     if (aba_use_warp<T>(n, B, flags)) return false;
-    return (flags & RD_ABA_FP64_UPDATE) ? true : B <= 16384;
+    return (flags & RD_ABA_FP64_UPDATE) ? true : B <= kAbaPairMost;
 }
 
 // Three warps per 32 instances (aba_tri.cuh): by flag, else for FP32 data where
@@ -249,9 +252,16 @@ inline bool aba_use_trio_f64(const rd_model *m, int B, int flags)
 }
 
 // Three lanes per instance (aba_trio.cuh): by flag, else for FP32 data with
-// double-float updates while the batch is resident at once, which is what the
-// split is for: four blocks per SM (thirty instances each, or twenty with the
-// double-float bias sweeps, where two such waves still win). Times in us on
+// double-float updates while four blocks per SM (thirty instances each, or twenty with
+// the double-float bias sweeps) hold the batch at once, with the latter in two waves.
+// Their records and constants leave room for three blocks from 90 links on (109 with the
+// double-float sweeps), which moves the line only where the two-warp kernel is the
+// alternative and close: us at B = 16384, two warps / three lanes: n = 95 with FP32 bias
+// sweeps (RD_ABA_FP32_BIAS) 421 / 444, n = 100 457 / 454, n = 128 591 / 585. With the
+// double-float sweeps, the mapping taken otherwise / three lanes: n = 108 888 / 765 at
+// 16384, 1071 / 1069 at 24320; n = 128 1056 / 889, 1260 / 1237; on the shortest chains
+// (RD_ABA_EXTENDED_BIAS) the second wave loses: n = 3 19.7 / 21.2 at 16384, 23.7 / 25.1 at
+// 22000; n = 5 33.0 / 34.3 at 16384; n = 10 79.6 / 82.5 at 24320. Times in us on
 // GB300, the mapping taken otherwise / three lanes: n = 7: 17.6 / 13.2 at B = 1024, 34.9 / 23.7 at
 // 18240, 35.7 / 38.1 at 24000; n = 64: 346 / 217 at 18240, 360 / 355 at 24000, 352 /
 // 440 at 32768; n = 100: 822 / 704 at 16384, 990 / 852 at 24000, 938 / 1197 at
@@ -273,7 +283,15 @@ inline bool aba_use_trio(const rd_model *m, int B, int flags, bool ext)
                                                                       : 0;
         if ((flags & RD_ABA_EXACT_MAPPING) || warps != replaced) return false;
     }
-    return m->n >= 3 && (long long)B <= (ext ? 160LL : 120LL) * rd_sm_count(m->device);
+    const int n = m->n;
+    const long long sms = rd_sm_count(m->device);
+    if (n < 3) return false;
+    if (ext) {
+        if (n <= 5 && B > 80 * sms && B <= kAbaPairMost) return false;
+        return B <= (n == 3 ? 136 : n >= 5 && n <= 11 ? 150 : 160) * sms;
+    }
+    if (n >= 90 && n < 100 && B > 90 * sms && B <= kAbaPairMost) return false;
+    return B <= 120 * sms;
 }
 
 template <typename T>

@@ -262,8 +262,8 @@ __device__ __forceinline__ To dcvt(From x)
     return DCvt<To>::from(x);
 }
 
-// A plain factor (the sine or cosine of a joint angle) beside values of type D:
-// an FP32 factor stays a float next to double-floats: its products take one
+// A plain factor (the sine or cosine of a joint angle) beside values of type D: an FP32
+// factor stays a float next to double-floats, where its products take one
 // multiply-add less.
 template <typename D>
 struct DScalar;
