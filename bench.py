@@ -99,10 +99,12 @@ FD_FLOP64_PER_LINK = 800
 FD_EXEC_FLOP32_PER_LINK = 257
 FD_EXEC_FLOP64_PER_LINK = 400
 # the default for FP32 data carries those FP64 operations in double-float
-# arithmetic on the FP32 pipe: FP32-pipe instructions executed per link, from
-# the FMA-pipe count of an ncu capture at n = 64, B = 16384 (99.7 M warp
-# instructions, 94% of all)
+# arithmetic on the FP32 pipe: FP32-pipe instructions executed per link (32 lanes a warp
+# instruction), from the FMA-pipe counts of ncu captures at n = 64, B = 16384: one thread
+# per instance 99.7 M warp instructions (94% of all), three lanes per instance, the
+# library's choice there and in mixed batches, 115.9 M (70% of all)
 FD_DF_EXEC_FP32_INST_PER_LINK = 3043
+FD_LANES_EXEC_FP32_INST_PER_LINK = 3537
 # FP32-pipe instructions per link of the double-float kernel for FP64 data
 # (RD_VARIANT_SERIAL_DF), from the FMA-pipe count of an ncu capture at n = 32,
 # B = 65536 (166.2 M warp instructions, 92% of all)
@@ -162,7 +164,7 @@ def parse_args():
     p.add_argument("--kernel-only",
                    choices=["f32", "f64", "f64df", "host", "vjp", "vjplane", "vjppair", "vjpsmem",
                             "aba", "aba64",
-                            "abawarp", "abapair", "abatri", "abatri1k", "fleet", "fleetpair",
+                            "abawarp", "abapair", "abatri", "abatri1k", "abatrio", "fleet", "fleetpair",
                             "fleettri64"],
                    default=None,
                    help="profiling case: W + K plain launches of one kernel, no JSON "
@@ -173,7 +175,8 @@ def parse_args():
                         "instances / state in shared memory; aba: forward dynamics n=64 B=16384 (double-float updates; "
                         "aba64: FP64 updates); abawarp: forward dynamics n=64 B=1024, one warp per "
                         "instance; abapair / abatri: forward dynamics n=64 B=16384, two / three "
-                        "warps per 32 instances; abatri1k: three warps at B=1024; fleet: 20000 "
+                        "warps per 32 instances; abatri1k: three warps at B=1024; abatrio: three "
+                        "lanes per instance, n=64 B=16384; fleet: 20000 "
                         "mixed requests; fleetpair: the same "
                         "with warp pairs for forward-dynamics chains from 65 links; fleettri64: "
                         "warp triples from 65 links, FP64 updates)")
@@ -454,10 +457,12 @@ def fd_section(torch, rd, chaingen, dev, dist, sampler, K):
             return time_calls(torch, call, steps, 3, dist, sampler) / steps
 
         raw[f"n{n}_B{B}"] = {"n": n, "B": B, "t64": timed(rd.RD_ABA_FP64_UPDATE), "tdf": timed(0)}
-    # the four mappings across batch sizes: microseconds [thread per instance,
-    # warp per instance (Sec. III-D scans), two warps per 32 instances, three
-    # warps per 32 instances, AUTO]; double-float updates at n = 16 and 64, FP64
-    # updates ("f64u") at n = 64
+        if rd.aba_last_mapping() == rd.RD_ABA_THREE_LANES:
+            raw[f"n{n}_B{B}"]["df_inst"] = FD_LANES_EXEC_FP32_INST_PER_LINK
+    # the mappings across batch sizes: microseconds [thread per instance, warp per
+    # instance (Sec. III-D scans), two warps per 32 instances, three warps per 32
+    # instances, AUTO (with double-float updates three lanes per instance)];
+    # double-float updates at n = 16 and 64, FP64 updates ("f64u") at n = 64
     xo = {}
     cases = [(n, Bx, 0) for n in (16, 64) for Bx in (256, 1024, 4096, 16384)]
     cases += [(64, Bx, rd.RD_ABA_FP64_UPDATE) for Bx in (256, 1024, 4096)]
@@ -471,7 +476,8 @@ def fd_section(torch, rd, chaingen, dev, dist, sampler, K):
         steps = max(3, min(K, 20))
         row = []
         for fl in (rd.RD_ABA_THREAD_PER_INSTANCE, rd.RD_ABA_WARP_PER_INSTANCE,
-                   rd.RD_ABA_TWO_WARPS, rd.RD_ABA_THREE_WARPS, 0):
+                   rd.RD_ABA_TWO_WARPS | rd.RD_ABA_EXACT_MAPPING,
+                   rd.RD_ABA_THREE_WARPS | rd.RD_ABA_EXACT_MAPPING, 0):
             t = time_calls(torch, lambda k: rd.aba(model, *x, workspace=ws, out=o, flags=fl | prec),
                            steps, 3, dist, sampler)
             row.append(t / steps * 1e6)
@@ -484,7 +490,8 @@ def fd_report(raw, pk):
     """frac: the kernel's executed FP32 and FP64 arithmetic at the two peaks
     (combined time) over the measured time; frac_alg: the same with the
     formulation's count (the method's work: 720 FP32 + 800 FP64 flop per link);
-    df_frac: FP32-pipe issue time of the double-float kernel's instructions."""
+    df_frac: FP32-pipe issue time of the instructions of the double-float kernel
+    that ran (df_inst per link)."""
     out = {}
     for name, r in raw.items():
         if name == "crossover_us":
@@ -493,7 +500,7 @@ def fd_report(raw, pk):
         nb = r["n"] * r["B"]
         t_exec = nb * (FD_EXEC_FLOP32_PER_LINK / pk.f32 + FD_EXEC_FLOP64_PER_LINK / pk.f64)
         t_alg = nb * (FD_FLOP32_PER_LINK / pk.f32 + FD_FLOP64_PER_LINK / pk.f64)
-        t_df = nb * FD_DF_EXEC_FP32_INST_PER_LINK / pk.i32
+        t_df = nb * r.get("df_inst", FD_DF_EXEC_FP32_INST_PER_LINK) / pk.i32
         out[name] = {"us": r["t64"] * 1e6, "frac": t_exec / r["t64"],
                      "frac_alg": t_alg / r["t64"], "df_us": r["tdf"] * 1e6,
                      "df_frac": t_df / r["tdf"]}
@@ -575,6 +582,10 @@ def uneven_section(torch, rd, chaingen, dev, dist, sampler, K, count=100000):
     steps = max(3, min(K, 20))
     raw = {"count": count, "joints": plan.total_joints, "groups": plan.groups,
            "fd_joints": int(np.sum(np.where(kinds == 1, plan.lengths, 0)))}
+    # this plan's double-float forward dynamics runs three lanes per request, unless the
+    # pick names warp pairs or triples
+    if not (tune_df >> 16) & 0xff:
+        raw["df_inst"] = FD_LANES_EXEC_FP32_INST_PER_LINK
     for name, (sc, tu) in (("persistent", (sched | f64, tune)),
                            ("per_group", (rd.RD_SCHED_PER_GROUP | f64, 0)),
                            ("df_persistent", (sched_df, tune_df))):
@@ -593,7 +604,7 @@ def uneven_report(raw, pk):
     n_id = raw["joints"] - n_fd
     t_id = n_id * max(ALGO_FLOP_PER_LINK / pk.f32, UNEVEN_ID_BYTES_PER_LINK / pk.hbm)
     t_fd = n_fd * (FD_EXEC_FLOP32_PER_LINK / pk.f32 + FD_EXEC_FLOP64_PER_LINK / pk.f64)
-    t_df = n_fd * FD_DF_EXEC_FP32_INST_PER_LINK / pk.i32
+    t_df = n_fd * raw.get("df_inst", FD_DF_EXEC_FP32_INST_PER_LINK) / pk.i32
     out = {}
     for name in ("persistent", "per_group", "df_persistent"):
         r = raw[name]
@@ -875,13 +886,14 @@ def run_kernel_only(args):
         x = [torch.from_numpy(st[k]).to(dev, torch.float32) for k in ("q", "qd", "qdd", "w")]
         for _ in range(calls):
             res = rd.rnea_vjp(model, *x, mode=mode)[0]
-    elif args.kernel_only in ("aba", "aba64", "abawarp", "abapair", "abatri", "abatri1k"):
+    elif args.kernel_only in ("aba", "aba64", "abawarp", "abapair", "abatri", "abatri1k", "abatrio"):
         flags = {"aba": rd.RD_ABA_THREAD_PER_INSTANCE,
                  "aba64": rd.RD_ABA_FP64_UPDATE | rd.RD_ABA_THREAD_PER_INSTANCE,
                  "abawarp": rd.RD_ABA_WARP_PER_INSTANCE,
-                 "abapair": rd.RD_ABA_TWO_WARPS,
-                 "abatri": rd.RD_ABA_THREE_WARPS,
-                 "abatri1k": rd.RD_ABA_THREE_WARPS}[args.kernel_only]
+                 "abapair": rd.RD_ABA_TWO_WARPS | rd.RD_ABA_EXACT_MAPPING,
+                 "abatri": rd.RD_ABA_THREE_WARPS | rd.RD_ABA_EXACT_MAPPING,
+                 "abatri1k": rd.RD_ABA_THREE_WARPS | rd.RD_ABA_EXACT_MAPPING,
+                 "abatrio": rd.RD_ABA_THREE_LANES}[args.kernel_only]
         Ba = 1024 if args.kernel_only in ("abawarp", "abatri1k") else 16384
         model = rd.Model(chaingen.make_chain(64, seed=chaingen.BASE_SEED))
         st = chaingen.make_states(Ba, 64, seed=6000, kinds=("q", "qd", "tau"))

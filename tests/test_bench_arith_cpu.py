@@ -76,3 +76,31 @@ def test_profile_traffic_is_reported_only_for_the_profiled_sources():
     else:
         assert got is None
     assert bench.recorded_traffic("no_such_profile") is None
+
+
+def test_executed_flops_of_the_origin_recursion_follow_the_per_link_parts():
+    """The count of the headline's kernel: a stored link's sin/cos, rotation products,
+    forward step (three rotated vectors, the next origin's acceleration, the joint's
+    terms), matrix W, bias wrench, carry and products; a re-derived link's inverse step."""
+    forward = 3 * 13 + 18 + 6
+    stored = 26 + 4 + forward + 21 + 60 + 44 + 4
+    assert (stored, stored + 84) == (222, 306)
+    for n, K in ((32, 32), (16, 16), (64, 12), (100, 0), (4, 4)):
+        want = K * stored + (n - K) * (stored + 84) - 38 - (84 if K < n else 0)
+        assert bench.origin_param_flops(n, K) == want
+
+
+def test_double_float_fractions_count_the_kernel_that_ran():
+    """Three lanes per instance where the library took them (115.9 M warp instructions on
+    the FMA pipe at n = 64, B = 16384), else one thread per instance (99.7 M)."""
+    pk = bench.Peaks(152, 2070.0)
+    per_link = [round(m * 1e6 * 32 / (64 * 16384)) for m in (115.905306, 99.697152)]
+    assert per_link == [bench.FD_LANES_EXEC_FP32_INST_PER_LINK, bench.FD_DF_EXEC_FP32_INST_PER_LINK]
+    raw = {"n": 64, "B": 16384, "t64": 6e-4, "tdf": 2e-4}
+    a = bench.fd_report({"x": dict(raw, df_inst=3537)}, pk)["x"]["df_frac"]
+    b = bench.fd_report({"x": raw}, pk)["x"]["df_frac"]
+    assert abs(a / b - 3537 / 3043) < 1e-12
+    fleet = {"joints": 1000, "fd_joints": 400, "count": 10,
+             **{k: {"t": 1e-3} for k in ("persistent", "per_group", "df_persistent")}}
+    one, lanes = (bench.uneven_report(r, pk)["df_persistent"]["frac"] for r in (fleet, dict(fleet, df_inst=3537)))
+    assert abs((lanes - one) * 1e-3 - 400 * (3537 - 3043) / pk.i32) < 1e-15
