@@ -200,7 +200,9 @@ constexpr int kAbaPairMost = 16384;
 // pair: n = 16: 1.25 at B = 1024, 1.04 at 16384, 0.80 at 65536; n = 64: 1.31 /
 // 1.17 / 0.76; n = 100: 1.90 / 1.20; FP64 updates: n = 64: 1.15 at 1024, 1.03 at
 // 16384, 1.05 at 65536; n = 100: 1.46 / 1.19) and the warp-per-instance mapping
-// does not apply.
+// does not apply. With double-float updates aba_use_trio comes first: this line and the
+// next one then serve chains of one or two links, and say which mapping a flag names
+// that three lanes replaced.
 template <typename T>
 bool aba_use_pair(int n, int B, int flags)
 {

@@ -31,10 +31,11 @@
 // solves. No thread spins on another.
 //
 // What bounds it: FP32 issue and, below one block per SM, the dependent chains of
-// the double-float updates (about 1.4 k instructions a link for ten instances, of
-// which 1.0 k on the FMA pipe; issue 65% with four warps per scheduler, no
-// instruction-fetch stalls: 0.09 per issue against 0.97 with one thread per
-// instance and 2.2 k straight-line instructions a link). Splitting by axis costs
+// the double-float updates (1.57 k warp instructions a link for ten instances, bias
+// included, of which 1.1 k on the FMA pipe; issue 65% with 3.1 warps per scheduler, few
+// instruction-fetch stalls: 0.09 per issue against 0.97 with two warps per 32
+// instances; one thread per instance runs 2.2 k straight-line instructions a link).
+// Splitting by axis costs
 // half as many instructions again per instance, but three times as many warps
 // run half the code each. us, GB300, FP32 data, two or three warps per 32
 // instances before / now: n = 7: B = 1024 17.6 / 13.2, 16384 28.8 / 23.7; n = 64:
@@ -47,7 +48,8 @@
 //   aba_pair.cuh; block of four warps, 0..2 with ten instances each, 3 with the
 //   bias of the thirty.
 //   Bias in double-float (chains beyond RD_ABA_EXTENDED_BIAS_LINKS): three lanes
-//   per instance there too; block of two warps for ten instances.
+//   per instance there too; block of four warps, 0 and 1 with ten instances each, 2
+//   and 3 with their bias.
 // Lanes 30 and 31 of a three-lane warp repeat the work of lanes 27 and 28 and
 // write nothing.
 //

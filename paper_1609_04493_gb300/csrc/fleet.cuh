@@ -248,8 +248,9 @@ __device__ __forceinline__ void fleet_request_pair(const FleetArgs<T, D> &a, int
 // bias sweeps; the inertias and the solves), or one warp doing both in turn. A
 // unit's bias sweeps run in double-float if any of its requests' groups of 32
 // asks for it, so a request's arithmetic depends on the plan alone, not on
-// the schedule. 20 000 requests of 6..100 links (4000 forward dynamics): 944 us with
-// one thread per request, 335 now; 1000 requests: 790 / 257; 100 000: 1150 / 594.
+// the schedule. us over one set of inputs, 6..100 links, one in five forward dynamics:
+// 20 000 requests 944 with one thread per request, 335 now (366 where the inputs change
+// from call to call); 1000 790 / 257; 100 000 1150 / 594.
 // Bound by the longest chains' dependent updates (100 links: 224 us alone).
 
 // Roles of a unit: one warp for both, or one of a pair.

@@ -401,7 +401,7 @@ int run_fleet(const rd_plan *p, const void *q, const void *qd, const void *in2, 
             // Three lanes per request. By default one pair of warps per block where every unit then has
             // a pair at once and the inverse-dynamics requests are few: the other
             // two warps would only take issue slots from the longest chains, which
-            // set the time (us, 128 threads / 64: 20 000 requests of 6..100 links 377 /
+            // set the time (us over one set of inputs, 128 threads / 64: 20 000 requests of 6..100 links 377 /
             // 335, of 6..64 184 / 158, 4000 of 8..40 91 / 85; 100 000 594 / 792, where
             // neither holds).
             const int units = (p->fd_count + rdyn::kTrioPerWarp - 1) / rdyn::kTrioPerWarp;

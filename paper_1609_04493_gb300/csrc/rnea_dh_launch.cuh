@@ -241,7 +241,8 @@ void dhp_default_kr(const rd_model *m, int B, int &K, int &RL, int &stages)
 // first four in registers, or eight for the longest chains in batches beyond two
 // waves (n = 31, B = 262144: 73 us against 79; n = 29, B = 49999: 17.9 against 15.7; n =
 // 13, B = 65536: 12.5 against 10.0: the unrolled code is fetched once a block); beyond
-// 32, dhp_default_k's K. us, joint-frame kernels with element loads / now: n = 7, B =
+// 32, dhp_default_k's K. us on the device over inputs that the L2 holds (n = 29 over
+// changing ones: 26.7 / 17.4 to 17.9), joint-frame kernels with element loads / now: n = 7, B =
 // 65536: 6.5 / 5.7; n = 13: 11.1 / 10.0; n = 29, B = 49999: 25.2 / 15.7; n = 63, B = 65536:
 // 108 / 47.5; n = 99: 123 / 73.5.
 template <int TRIG>

@@ -368,7 +368,7 @@ int dispatch(const rd_model *m, int B, const void *q, const void *qd, const void
     }
     if (variant == RD_VARIANT_AUTO) {
         // Sweep on GB300 at B = 65536 (modes x block sizes x stored links):
-        // (now for tuned calls, FP64 also n > 108)
+        // (now for tuned calls, FP32 rows of one or two links, FP64 n > 108)
         // per-link state in shared memory wins while it is small (FP32 n <= 32,
         // FP64 n <= 16); FP64 up to n = 32 keeps part of it in registers; up to
         // n = 64 the first links keep their state and the rest are re-derived;

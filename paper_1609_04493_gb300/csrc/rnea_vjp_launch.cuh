@@ -276,7 +276,9 @@ int launch_vjp_any(const rd_model *m, int B, const void *q, const void *qd, cons
                                                  split, lanes, s);
     }
     // Rows of other lengths and alignments: the common-normal kernel for FP64 (fewer FP64
-    // instructions: n = 7, B = 8192: 98 us against 107; 29: 403 against 455) and, in FP32,
+    // instructions: 0.81 to 0.96 of the joint-frame kernel's time at 31 lengths from 1 to
+    // 128, B = 1 to 65536, re-deriving or stored; n = 7, B = 8192: 98 us against 107; 29:
+    // 403 against 455) and, in FP32,
     // where its arithmetic outweighs the shifts of its loads (joint frames / this, B =
     // 8192 and 65536: n = 7: 7.7 / 8.9, 13.3 / 16.1; 14: 12.4 / 12.0, 26.0 / 28.3; 19: 17.6
     // / 14.2, 36.2 / 37.3; 21: 19.1 / 14.7, 40.8 / 39.8; 25: 21.8 / 16.3, 49.0 / 43.2; 63 at
